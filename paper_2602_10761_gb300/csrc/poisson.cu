@@ -37,6 +37,14 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Mixed-radix (4, 2, 3) Stockham plan for one transform length.
+struct FftPlan {
+    int n = 0;
+    int npass = 0;
+    int radix[24];
+    void* tw = nullptr;      // device table, n entries of cplx<R>: exp(-2 pi i e / n)
+};
+
 bool make_plan_radices(int n, FftPlan& p) {
     p.n = n;
     p.npass = 0;
@@ -45,22 +53,6 @@ bool make_plan_radices(int n, FftPlan& p) {
     while (m % 2 == 0) { p.radix[p.npass++] = 2; m /= 2; }
     while (m % 3 == 0) { p.radix[p.npass++] = 3; m /= 3; }
     return m == 1 && p.npass <= 24;
-}
-
-template <class R>
-tribo_status make_plan(int n, FftPlan& p) {
-    if (!make_plan_radices(n, p)) {
-        set_last_error("FFT length " + std::to_string(n) + " is not 2^a 3^b");
-        return TRIBO_ERR_UNSUPPORTED;
-    }
-    std::vector<cplx<R>> tw(n);
-    for (int e = 0; e < n; ++e) {
-        double a = 2.0 * M_PI * (double)e / (double)n;
-        tw[e] = cplx<R>{(R)std::cos(a), (R)(-std::sin(a))};
-    }
-    TRIBO_CUDA(cudaMalloc(&p.tw, sizeof(cplx<R>) * n));
-    TRIBO_CUDA(cudaMemcpy(p.tw, tw.data(), sizeof(cplx<R>) * n, cudaMemcpyHostToDevice));
-    return TRIBO_OK;
 }
 
 // In-place radix-r DFT of y[0..r) with direction sgn (-1 forward, +1 inverse).
@@ -297,87 +289,6 @@ size_t smem_inv_x(int nx, int lpb) { return sizeof(cplx<R>) * 2 * (size_t)lpb * 
 template <class R> int lines_per_block() { return sizeof(R) == 4 ? 4 : 2; }
 template <class R> int z_tile() { return sizeof(R) == 4 ? 8 : 4; }
 
-// The per-function dynamic shared-memory limit is process-wide state shared by
-// every context on the device, so it is raised to the device's opt-in maximum
-// (never lowered to one context's need); each launch still requests only what
-// it uses.
-template <class R>
-tribo_status setup_kernels(tribo_ctx* c) {
-    const int lpb = lines_per_block<R>();
-    int dev = 0, optin = 0;
-    TRIBO_CUDA(cudaGetDevice(&dev));
-    TRIBO_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    const size_t need = std::max({smem_fwd_x<R>(c->nx, lpb), smem_inv_x<R>(c->nx, lpb),
-                                  sizeof(cplx<R>) * 2 * z_tile<R>() * c->nz});
-    if (need > (size_t)optin) {
-        set_last_error("grid needs more shared memory per block than the device offers");
-        return TRIBO_ERR_UNSUPPORTED;
-    }
-    TRIBO_CUDA(cudaFuncSetAttribute(k_fwd_x<R, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_fwd_x<R, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_inv_x<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_fft_z<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    return TRIBO_OK;
-}
-
-template <class R>
-tribo_status solve_impl(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src, double* phi,
-                        void* Evoid) {
-    const int nx = c->nx, ny = c->ny, nz = c->nz, nxh = c->nxh;
-    cplx<R>* S = (cplx<R>*)c->S;
-    cplx<R>* F = (cplx<R>*)c->F;
-    const int lpb = lines_per_block<R>();
-    const int mt = z_tile<R>();
-    {
-        const int nlines = ny * nz;
-        dim3 grid((nlines + lpb - 1) / lpb);
-        phase_begin(c, PH_FWD_X);
-        if (src_f64 && sizeof(R) == 4)
-            k_fwd_x<R, double><<<grid, kThreads, smem_fwd_x<R>(nx, lpb), c->stream>>>(
-                (double*)src, scale, zero_src ? 1 : 0, S, nx, ny, nlines, nxh, c->plan_x, lpb);
-        else
-            k_fwd_x<R, R><<<grid, kThreads, smem_fwd_x<R>(nx, lpb), c->stream>>>(
-                (R*)src, scale, zero_src ? 1 : 0, S, nx, ny, nlines, nxh, c->plan_x, lpb);
-        TRIBO_LAUNCHED(c);
-    }
-    {
-        dim3 grid(ny, (nxh + mt - 1) / mt, 1);
-        phase_begin(c, PH_FWD_Z);
-        k_fft_z<R><<<grid, kThreads, sizeof(cplx<R>) * 2 * mt * nz, c->stream>>>(
-            S, nz, ny, nxh, mt, c->plan_z, (R)-1, 0);
-        TRIBO_LAUNCHED(c);
-    }
-    const int want_phi = phi != nullptr ? 1 : 0;
-    const int nf = 3 + want_phi;
-    {
-        const int np = nz * nxh;
-        double2* W = (double2*)c->W;
-        double* Wc = (double*)(W + (size_t)ny * np);
-        phase_begin(c, PH_SOLVE_Y);
-        k_solve_y<R><<<(np + 127) / 128, 128, 0, c->stream>>>(S, F, W, Wc, c->d_ycoef, c->d_lamx, c->d_lamz,
-                                                             c->d_sinx, c->d_sinz, c->d_ey, ny, nz, nxh,
-                                                             want_phi);
-        TRIBO_LAUNCHED(c);
-    }
-    {
-        const size_t fstride = (size_t)nz * (ny + 2) * nxh;
-        dim3 grid(ny + 2, (nxh + mt - 1) / mt, nf);
-        phase_begin(c, PH_INV_Z);
-        k_fft_z<R><<<grid, kThreads, sizeof(cplx<R>) * 2 * mt * nz, c->stream>>>(
-            F, nz, ny + 2, nxh, mt, c->plan_z, (R)1, fstride);
-        TRIBO_LAUNCHED(c);
-    }
-    {
-        const int nlines = nz * (ny + 2);
-        dim3 grid((nlines + lpb - 1) / lpb);
-        phase_begin(c, PH_INV_X);
-        k_inv_x<R><<<grid, kThreads, smem_inv_x<R>(nx, lpb), c->stream>>>(
-            F, (R*)Evoid, phi, nx, ny, nz, nxh, c->plan_x, lpb, nf);
-        TRIBO_LAUNCHED(c);
-    }
-    return TRIBO_OK;
-}
-
 }  // namespace
 
 tribo_status poisson_setup(tribo_ctx* c) {
@@ -442,25 +353,7 @@ tribo_status poisson_setup(tribo_ctx* c) {
     const size_t csz = 2 * rsz;
     TRIBO_CUDA(cudaMalloc(&c->S, csz * (size_t)nz * ny * nxh));
     TRIBO_CUDA(cudaMalloc(&c->F, csz * 4 * (size_t)nz * (ny + 2) * nxh));
-    tribo_status st;
-    c->fast = poisson_fast_supported(nx, nz);
-    if (c->fast) {
-        st = poisson_fast_setup(c);
-        if (st == TRIBO_OK) return TRIBO_OK;
-        if (st != TRIBO_ERR_UNSUPPORTED) return st;
-        poisson_fast_free(c);
-        c->d_ytab = c->W2 = c->d_twx = c->d_twz = nullptr;
-        c->fast = false;
-    }
-    TRIBO_CUDA(cudaMalloc(&c->W, (sizeof(double2) + sizeof(double)) * (size_t)ny * nz * nxh));
-    if (c->prec == TRIBO_FP64) {
-        if ((st = make_plan<double>(nx, c->plan_x)) != TRIBO_OK) return st;
-        if ((st = make_plan<double>(nz, c->plan_z)) != TRIBO_OK) return st;
-        return setup_kernels<double>(c);
-    }
-    if ((st = make_plan<float>(nx, c->plan_x)) != TRIBO_OK) return st;
-    if ((st = make_plan<float>(nz, c->plan_z)) != TRIBO_OK) return st;
-    return setup_kernels<float>(c);
+    return poisson_fast_setup(c);
 }
 
 tribo_status poisson_free(tribo_ctx* c) {
@@ -472,19 +365,8 @@ tribo_status poisson_free(tribo_ctx* c) {
     cudaFree(c->d_ey);
     cudaFree(c->S);
     cudaFree(c->F);
-    cudaFree(c->W);
-    cudaFree(c->plan_x.tw);
-    cudaFree(c->plan_z.tw);
     poisson_fast_free(c);
     return TRIBO_OK;
-}
-
-tribo_status poisson_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
-                           double* phi, void* E) {
-    if (c->fast) return poisson_fast_solve(c, src, src_f64, scale, zero_src, phi, E);
-    if (!E) E = c->E_lat;       // the generic passes always form the field
-    if (c->prec == TRIBO_FP64) return solve_impl<double>(c, src, true, scale, zero_src, phi, E);
-    return solve_impl<float>(c, src, src_f64, scale, zero_src, phi, E);
 }
 
 }  // namespace tribo
@@ -639,7 +521,7 @@ tribo_status noalloc_solve(const tribo_grid* g, double eps, const double* rho, d
     const int nx = g->nx, ny = g->ny, nz = g->nz, nxh = nx / 2 + 1;
     const int lpb = lines_per_block<R>();
     const int mt = z_tile<R>();
-    // the kernels' shared memory, as the context path checks it (poisson setup_kernels)
+    // the kernels' shared memory, against the device
     const size_t need = std::max({smem_fwd_x<R>(nx, lpb), smem_inv_x<R>(nx, lpb), sizeof(cplx<R>) * 2 * mt * nz});
     if (need > (size_t)smem_max) {
         set_last_error("tribo_poisson_noalloc: grid needs more shared memory per block than the device offers");

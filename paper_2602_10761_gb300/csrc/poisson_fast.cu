@@ -1,9 +1,10 @@
-// Poisson solve and E field, bandwidth-oriented path for compile-time
-// transform lengths (nx/2 and nz in {2, 3, 4, 6, 8, 12, ..., 384, 512}).
-//
-// Same discretisation and result as the generic path in poisson.cu (Sec. 2.2
-// Poisson equation with grounded walls, second-order finite volumes of
-// Sec. 3.1, E = -grad(phi) with Gauss-linear E_y and central E_x, E_z), but:
+// Poisson solve and E field of a context (Sec. 2.2 Poisson equation with
+// grounded walls, second-order finite volumes of Sec. 3.1, E = -grad(phi) with
+// Gauss-linear E_y and central E_x, E_z; the discretisation is described in
+// poisson.cu).  Every supported length 2^a 3^b has compiled transforms and
+// tabulated y factors (the field of a 288 x 145 x 162 grid in mixed precision:
+// 201 us; 1167 us with shared-memory Stockham passes and an FP64 Thomas sweep
+// with a division per row):
 //  * the x transforms are real: a length-nx/2 complex FFT of the packed line
 //    plus the split step (half the work and shared memory);
 //  * the y factorisation depends only on lam = lam_x + lam_z, so the factors
@@ -508,116 +509,6 @@ tribo_status dispatch_attr_fused(int m, int nz, int optin) {
     return TRIBO_ERR_UNSUPPORTED;
 }
 
-template <class R, int M, class QT>
-void launch_xfwd(tribo_ctx* c, QT* src, const double* scale, bool zero) {
-    constexpr int LPB = fft::FourStep<M, kThreads>::W;
-    const int nlines = c->ny * c->nz;
-    (void)launch_pdl(k_xfwd4<R, M, QT>, dim3((nlines + LPB - 1) / LPB), dim3(kThreads), xfwd_smem<R, M>(), c->stream,
-                     src, scale, zero ? 1 : 0, (cplx<R>*)c->S, c->ny, nlines, (const cplx<R>*)c->d_twx,
-                     (const FastTab<R>*)nullptr);
-}
-template <class R, int M>
-void launch_xinv(tribo_ctx* c, void* E, double* phi) {
-    constexpr int LPB = fft::FourStep<M, kThreads>::W;
-    const int nlines = c->nz * (c->ny + 2);
-    const size_t fstride = (size_t)c->nz * (c->ny + 2) * c->nxh;
-    static int occ = 0;
-    const int g = wave_blocks(k_xinv4<R, M>, xinv_smem<R, M>(), c->num_sms, (nlines + LPB - 1) / LPB, &occ);
-    k_xinv4<R, M><<<g, kThreads, xinv_smem<R, M>(), c->stream>>>(
-        (const cplx<R>*)c->F, (R*)E, phi, c->ny, c->nz, fstride, c->d_sinx, (const cplx<R>*)c->d_twx,
-        phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, (R)(1.0 / ((double)c->nx * (double)c->nz)),
-        (size_t)c->nz * (c->ny + 2) * c->nx, nullptr);
-}
-template <class R, int NZ>
-void launch_zfwd(tribo_ctx* c) {
-    constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    static int occ = 0;
-    const int grid = wave_blocks(k_zfwd4<R, NZ>, zfwd_smem<R, NZ>(), c->num_sms,
-                                 (int64_t)c->ny * ((c->nxh + W - 1) / W), &occ);
-    (void)launch_pdl(k_zfwd4<R, NZ>, dim3(grid), dim3(kThreads), zfwd_smem<R, NZ>(), c->stream, (cplx<R>*)c->S, c->ny,
-                     c->nxh, (const cplx<R>*)c->d_twz, (const FastTab<R>*)nullptr);
-}
-template <class R, int NZ>
-void launch_zinv(tribo_ctx* c, bool phi_only) {
-    constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    static int occ = 0;
-    const int grid = wave_blocks(k_zinv4<R, NZ>, zinv_smem<R, NZ>(), c->num_sms,
-                                 (int64_t)(c->ny + 2) * ((c->nxh + W - 1) / W), &occ);
-    const size_t fstride = (size_t)c->nz * (c->ny + 2) * c->nxh;
-    k_zinv4<R, NZ><<<grid, kThreads, zinv_smem<R, NZ>(), c->stream>>>(
-        (const cplx<R>*)c->S, (cplx<R>*)c->F, c->ny, c->nxh, fstride, c->d_sinz, (const cplx<R>*)c->d_twz,
-        phi_only ? 1 : 0, nullptr);
-}
-template <class R, int NZ>
-tribo_status attr_z(int optin) {
-    if (zfwd_smem<R, NZ>() > (size_t)optin || zinv_smem<R, NZ>() > (size_t)optin) return TRIBO_ERR_UNSUPPORTED;
-    TRIBO_CUDA(cudaFuncSetAttribute(k_zfwd4<R, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_zinv4<R, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    return TRIBO_OK;
-}
-template <class R, int M>
-tribo_status attr_x(int optin) {
-    if (xfwd_smem<R, M>() > (size_t)optin || xinv_smem<R, M>() > (size_t)optin) return TRIBO_ERR_UNSUPPORTED;
-    TRIBO_CUDA(cudaFuncSetAttribute(k_xfwd4<R, M, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_xfwd4<R, M, double>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_xinv4<R, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    return TRIBO_OK;
-}
-
-template <class R, class QT>
-bool dispatch_xfwd(tribo_ctx* c, QT* src, const double* scale, bool zero) {
-    switch (c->nx / 2) {
-#define CASE(N) case N: launch_xfwd<R, N, QT>(c, src, scale, zero); return true;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: return false;
-    }
-}
-template <class R>
-bool dispatch_xinv(tribo_ctx* c, void* E, double* phi) {
-    switch (c->nx / 2) {
-#define CASE(N) case N: launch_xinv<R, N>(c, E, phi); return true;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: return false;
-    }
-}
-template <class R>
-bool dispatch_zfwd(tribo_ctx* c) {
-    switch (c->nz) {
-#define CASE(N) case N: launch_zfwd<R, N>(c); return true;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: return false;
-    }
-}
-template <class R>
-bool dispatch_zinv(tribo_ctx* c, bool phi_only) {
-    switch (c->nz) {
-#define CASE(N) case N: launch_zinv<R, N>(c, phi_only); return true;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: return false;
-    }
-}
-template <class R>
-tribo_status dispatch_attr(int nx, int nz, int optin) {
-    tribo_status st = TRIBO_ERR_UNSUPPORTED;
-    switch (nz) {
-#define CASE(N) case N: st = attr_z<R, N>(optin); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: break;
-    }
-    if (st) return st;
-    switch (nx / 2) {
-#define CASE(N) case N: return attr_x<R, N>(optin);
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: return TRIBO_ERR_UNSUPPORTED;
-    }
-}
-
 // tw[e] = exp(-2 pi i e / n), e < n; for the x length (with_inner) also the four-step's inner
 // twiddles of M = n/2 = N1 N2 laid out by thread: tw[n + k1 N2 + r] = W_M^(r k1), so that the
 // 16 threads of a column read 16 consecutive values (the lookup tw[2 r k1] hits one shared-memory
@@ -657,12 +548,14 @@ tribo_status solve_fast(tribo_ctx* c, void* src, bool src_f64, const double* sca
     // tasks would hold SMs the other channels' passes could use)
     // (the potential-only solves of the adjoint also keep the split passes)
     const bool fused = c->ring != nullptr && !c->in_batch && E != nullptr;
+    const PassGrid<R> g{c->nx, ny, nz, nxh, c->num_sms, c->stream};
+    const cplx<R>* twx = (const cplx<R>*)c->d_twx;
+    const cplx<R>* twz = (const cplx<R>*)c->d_twz;
     phase_begin(c, PH_FWD_X);
-    if (src_f64) dispatch_xfwd<R, double>(c, (double*)src, scale, zero_src);
-    else dispatch_xfwd<R, R>(c, (R*)src, scale, zero_src);
+    xfwd_launch<R>(g, src, src_f64, scale, zero_src, (cplx<R>*)c->S, twx);
     TRIBO_LAUNCHED(c);
     phase_begin(c, PH_FWD_Z);
-    dispatch_zfwd<R>(c);
+    zfwd_launch<R>(g, (cplx<R>*)c->S, twz);
     TRIBO_LAUNCHED(c);
     const size_t fstride = (size_t)nz * (ny + 2) * nxh;
     const int ni = (nz / 2 + 1) * nxh;
@@ -696,17 +589,15 @@ tribo_status solve_fast(tribo_ctx* c, void* src, bool src_f64, const double* sca
         return TRIBO_OK;
     }
     phase_begin(c, PH_INV_Z);
-    dispatch_zinv<R>(c, E == nullptr);
+    zinv_launch<R>(g, (const cplx<R>*)c->S, (cplx<R>*)c->F, c->d_sinz, twz, E == nullptr);
     TRIBO_LAUNCHED(c);
     phase_begin(c, PH_INV_X);
-    dispatch_xinv<R>(c, E, phi);
+    xinv_launch<R>(g, (const cplx<R>*)c->F, (R*)E, phi, c->d_sinx, twx);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }
 
 }  // namespace
-
-bool poisson_fast_supported(int nx, int nz) { return nx >= 4 && nx % 2 == 0 && fast_len(nx / 2) && fast_len(nz); }
 
 tribo_status poisson_fast_setup(tribo_ctx* c) {
     const int nx = c->nx, ny = c->ny, nz = c->nz, nxh = c->nxh;
@@ -825,10 +716,14 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
     }
     if (c->prec == TRIBO_FP64) {
         if ((st = twiddles<double>(nx, &c->d_twx, true)) || (st = twiddles<double>(nz, &c->d_twz))) return st;
-        return dispatch_attr<double>(nx, nz, optin);
+        if ((st = zpass_attr<double>(nz, optin))) return st;
+        return xpass_attr<double>(nx / 2, optin);
     }
     if ((st = twiddles<float>(nx, &c->d_twx, true)) || (st = twiddles<float>(nz, &c->d_twz))) return st;
-    if (ysolve_twist_smem(ny) > (size_t)optin) return TRIBO_ERR_UNSUPPORTED;
+    if (ysolve_twist_smem(ny) > (size_t)optin) {
+        set_last_error("grid needs more shared memory per block than the device offers");
+        return TRIBO_ERR_UNSUPPORTED;
+    }
     TRIBO_CUDA(cudaFuncSetAttribute(k_ysolve_twist<kTwistC>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     TRIBO_CUDA(cudaFuncSetAttribute(k_ysolve_twist<kTwistC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     optin));
@@ -837,7 +732,8 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
     TRIBO_CUDA(cudaFuncSetAttribute((k_ysolve_twist<kTwistC2, false, false, 2>),
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     c->smem_optin = optin;
-    return dispatch_attr<float>(nx, nz, optin);
+    if ((st = zpass_attr<float>(nz, optin))) return st;
+    return xpass_attr<float>(nx / 2, optin);
 }
 
 void poisson_fast_free(tribo_ctx* c) {
@@ -854,8 +750,8 @@ void poisson_fast_free(tribo_ctx* c) {
     c->d_ytab = c->W2 = c->d_twx = c->d_twz = c->d_yads = c->d_yec = c->ring = c->d_pipe = nullptr;
 }
 
-tribo_status poisson_fast_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
-                                double* phi, void* E) {
+tribo_status poisson_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
+                           double* phi, void* E) {
     if (c->prec == TRIBO_FP64) return solve_fast<double>(c, src, true, scale, zero_src, phi, E);
     return solve_fast<float>(c, src, src_f64, scale, zero_src, phi, E);
 }

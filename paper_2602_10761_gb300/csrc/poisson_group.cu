@@ -19,112 +19,15 @@ struct Group {
     FastTab<float>* d_tab = nullptr;
 };
 
-template <int M>
-void group_xfwd(const Group& g, cudaStream_t st) {
-    constexpr int LPB = fft::FourStep<M, kThreads>::W;
-    const int nlines = g.ny * g.nz;
-    k_xfwd4<float, M, double, true><<<dim3((nlines + LPB - 1) / LPB, g.n), kThreads, xfwd_smem<float, M>(), st>>>(
-        nullptr, nullptr, 1, nullptr, g.ny, nlines, nullptr, g.d_tab);
-}
-template <int NZ>
-void group_zfwd(const Group& g, cudaStream_t st) {
-    constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    static int occ = 0;
-    const int64_t tiles = (int64_t)g.ny * ((g.nxh + W - 1) / W);
-    const int gx = std::max(1, wave_blocks(k_zfwd4<float, NZ, true>, zfwd_smem<float, NZ>(), g.num_sms, tiles, &occ) / g.n);
-    k_zfwd4<float, NZ, true><<<dim3(gx, g.n), kThreads, zfwd_smem<float, NZ>(), st>>>(nullptr, g.ny, g.nxh, nullptr, g.d_tab);
-}
-template <int NZ>
-void group_zinv(const Group& g, cudaStream_t st) {
-    constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    static int occ = 0;
-    const int64_t tiles = (int64_t)(g.ny + 2) * ((g.nxh + W - 1) / W);
-    const int gx = std::max(1, wave_blocks(k_zinv4<float, NZ, true>, zinv_smem<float, NZ>(), g.num_sms, tiles, &occ) / g.n);
-    const size_t fstride = (size_t)g.nz * (g.ny + 2) * g.nxh;
-    k_zinv4<float, NZ, true><<<dim3(gx, g.n), kThreads, zinv_smem<float, NZ>(), st>>>(nullptr, nullptr, g.ny, g.nxh,
-                                                                              fstride, nullptr, nullptr, 0, g.d_tab);
-}
-template <int M>
-void group_xinv(const Group& g, cudaStream_t st) {
-    constexpr int LPB = fft::FourStep<M, kThreads>::W;
-    static int occ = 0;
-    const int nlines = g.nz * (g.ny + 2);
-    const int gx = std::max(1, wave_blocks(k_xinv4<float, M, true>, xinv_smem<float, M>(), g.num_sms,
-                                           (nlines + LPB - 1) / LPB, &occ) / g.n);
-    const size_t fstride = (size_t)g.nz * (g.ny + 2) * g.nxh;
-    k_xinv4<float, M, true><<<dim3(gx, g.n), kThreads, xinv_smem<float, M>(), st>>>(
-        nullptr, nullptr, nullptr, g.ny, g.nz, fstride, nullptr, nullptr, 0, 1,
-        (float)(1.0 / ((double)g.nx * (double)g.nz)), (size_t)g.nz * (g.ny + 2) * g.nx, g.d_tab);
-}
 void group_ysolve(const Group& g, cudaStream_t st) {
     const int64_t nblk = ((int64_t)g.nz * g.nxh + 127) / 128;
     k_ysolve_twist<kTwistC, true, true><<<dim3((unsigned)nblk, g.n), 128, ysolve_twist_smem(g.ny), st>>>(
         nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, g.ny, g.nz, g.nxh, g.d_tab);
 }
 
-bool group_dispatch(const Group& g, cudaStream_t st) {
-    bool ok = true;
-    switch (g.nx / 2) {
-#define CASE(N) case N: group_xfwd<N>(g, st); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: ok = false;
-    }
-    switch (g.nz) {
-#define CASE(N) case N: group_zfwd<N>(g, st); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: ok = false;
-    }
-    group_ysolve(g, st);
-    switch (g.nz) {
-#define CASE(N) case N: group_zinv<N>(g, st); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: ok = false;
-    }
-    switch (g.nx / 2) {
-#define CASE(N) case N: group_xinv<N>(g, st); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: ok = false;
-    }
-    return ok;
-}
-
-// the group instantiations' shared-memory limits (the device's opt-in maximum)
-template <int M>
-tribo_status group_attr_x(int optin) {
-    if (xfwd_smem<float, M>() > (size_t)optin || xinv_smem<float, M>() > (size_t)optin) return TRIBO_ERR_UNSUPPORTED;
-    TRIBO_CUDA(cudaFuncSetAttribute(k_xfwd4<float, M, double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_xinv4<float, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    return TRIBO_OK;
-}
-template <int NZ>
-tribo_status group_attr_z(int optin) {
-    if (zfwd_smem<float, NZ>() > (size_t)optin || zinv_smem<float, NZ>() > (size_t)optin) return TRIBO_ERR_UNSUPPORTED;
-    TRIBO_CUDA(cudaFuncSetAttribute(k_zfwd4<float, NZ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_zinv4<float, NZ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    return TRIBO_OK;
-}
 tribo_status group_attr(const Group& g) {
-    tribo_status st = TRIBO_ERR_UNSUPPORTED;
-    switch (g.nx / 2) {
-#define CASE(N) case N: st = group_attr_x<N>(g.smem_optin); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: break;
-    }
-    if (st) return st;
-    st = TRIBO_ERR_UNSUPPORTED;
-    switch (g.nz) {
-#define CASE(N) case N: st = group_attr_z<N>(g.smem_optin); break;
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        default: break;
-    }
-    if (st) return st;
+    tribo_status st;
+    if ((st = xpass_attr<float>(g.nx / 2, g.smem_optin)) || (st = zpass_attr<float>(g.nz, g.smem_optin))) return st;
     if (ysolve_twist_smem(g.ny) > (size_t)g.smem_optin) return TRIBO_ERR_UNSUPPORTED;
     TRIBO_CUDA(cudaFuncSetAttribute((k_ysolve_twist<kTwistC, true, true>),
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_optin));
@@ -133,7 +36,7 @@ tribo_status group_attr(const Group& g) {
 
 }  // namespace
 
-bool poisson_group_ok(const tribo_ctx* c) { return c->fast && c->prec == TRIBO_MIXED; }
+bool poisson_group_ok(const tribo_ctx* c) { return c->prec == TRIBO_MIXED; }
 
 tribo_status poisson_group_create(tribo_ctx* const* chans, int n, void** out) {
     *out = nullptr;
@@ -143,7 +46,7 @@ tribo_status poisson_group_create(tribo_ctx* const* chans, int n, void** out) {
     for (int i = 0; i < n; ++i) {
         tribo_ctx* c = chans[i];
         if (!poisson_group_ok(c) || c->nx != c0->nx || c->ny != c0->ny || c->nz != c0->nz) {
-            set_last_error("a Poisson group needs mixed-precision channels of one compiled-length grid");
+            set_last_error("a Poisson group needs mixed-precision channels of one grid");
             return TRIBO_ERR_ARG;
         }
         const int ni = (c->nz / 2 + 1) * c->nxh;
@@ -188,10 +91,12 @@ tribo_status poisson_group_create(tribo_ctx* const* chans, int n, void** out) {
 
 tribo_status poisson_group_solve(void* grp, cudaStream_t stream, int64_t* launches) {
     const Group* g = static_cast<const Group*>(grp);
-    if (!group_dispatch(*g, stream)) {
-        set_last_error("Poisson group: length without a compiled transform");
-        return TRIBO_ERR_UNSUPPORTED;
-    }
+    const PassGrid<float> pg{g->nx, g->ny, g->nz, g->nxh, g->num_sms, stream, g->d_tab, g->n};
+    xfwd_launch<float>(pg, nullptr, true, nullptr, true, nullptr, nullptr);
+    zfwd_launch<float>(pg, nullptr, nullptr);
+    group_ysolve(*g, stream);
+    zinv_launch<float>(pg, nullptr, nullptr, nullptr, nullptr, false);
+    xinv_launch<float>(pg, nullptr, nullptr, nullptr, nullptr, nullptr);
     TRIBO_CUDA(cudaGetLastError());
     if (launches) *launches += 5;
     return TRIBO_OK;

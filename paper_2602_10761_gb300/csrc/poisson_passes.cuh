@@ -1,9 +1,10 @@
 // The split passes of the Poisson solve for compile-time transform lengths
 // (x forward, z forward, y solve, z inverse, x inverse; Sec. 2.2 Poisson
 // equation, second-order finite volumes of Sec. 3.1): kernels, their shared
-// memory sizes and the list of compiled lengths.  Included by poisson_fast.cu
-// (single channels, the fused inverse pipeline) and poisson_group.cu (groups
-// of channels solved together).
+// memory sizes and the list of compiled lengths.  The x and z transforms are
+// instantiated and launched by poisson_x32/x64/z32/z64.cu (one translation
+// unit per direction and precision, so that they compile side by side), the y
+// solves by poisson_fast.cu and poisson_group.cu.
 #pragma once
 
 #include <algorithm>
@@ -18,6 +19,15 @@ namespace tribo {
 namespace {
 
 constexpr int kThreads = 256;
+
+// resident blocks per SM that leave a transform of length N room for the larger factor's values
+// in registers (2 sizeof(R)/4 registers a value, and as many for the pass in flight): 64 registers
+// a thread hold 16 FP32 or 8 FP64 values, 128 hold twice as many
+template <class R, int N>
+constexpr int fft_min_blocks() {
+    return fft::FourStep<N, kThreads>::N2 * (int)sizeof(R) <= 64 ? 4
+           : fft::FourStep<N, kThreads>::N2 * (int)sizeof(R) <= 128 ? 2 : 1;
+}
 
 // ---------------------------------------------------------------- double-single
 struct ds {
@@ -45,31 +55,6 @@ __device__ __forceinline__ ds ds_mul(ds a, ds b) {
 __device__ __forceinline__ ds ds_neg(ds a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ float ds_f(ds a) { return a.hi + a.lo; }
 
-// ---------------------------------------------------------------- channel tables
-// The split passes also run for a group of channels with the same grid in
-// one launch each (a batch's channels, blockIdx.y = channel): the kTab
-// instantiation of a pass takes its channel's arrays from tab[blockIdx.y]
-// instead of its pointer arguments (a separate instantiation, so that the
-// single-channel passes keep their pointers in the parameter space and their
-// register budgets).
-template <class R>
-struct FastTab {
-    void* src;                  // FP64 cell charge sums (forward x source)
-    const double* scale;        // per-row RHS factor
-    cplx<R>* S;                 // spectrum
-    cplx<R>* F;                 // field spectra (the E_y spectrum at F + fstride)
-    R* E;                       // field lattice
-    const cplx<R>* twx;
-    const cplx<R>* twz;
-    const double* sinx;
-    const double* sinz;
-    const float2* tinv;         // y solve (mixed): 1/pivot, c' (double-single), sub-diagonal, E_y coefficients
-    const float2* tcp;
-    const float2* yads;         // y couplings (twisted solve: a_j, c_j), E_y coefficients, chunk checkpoints
-    const float4* yec;
-    float4* yck;
-};
-
 // ---------------------------------------------------------------- x forward
 // Thread group (line, r) per line (k, j) of the charge-sum array:
 // z_n = x_2n + i x_2n+1 (scaled to -rho/eps), Z = FFT_M(z) by the register
@@ -77,10 +62,10 @@ struct FastTab {
 // m = 0..M.  Each thread zeroes the charge sums it has read.  The source has
 // type QT: the FP64 cell charge sums (or a caller's FP64 density), rounded to
 // R as they are read, or the adjoint's R-typed charge adjoint.
-// six resident blocks (40 registers) where the length fits them without spilling: FP32 up to
-// M = 192 (76 -> 75.8 us at 384x256x256); one otherwise
+// six resident blocks (40 registers) where the length fits them without spilling: FP32 factors up
+// to 16 (76 -> 75.8 us at 384x256x256); one otherwise
 template <class R, int M>
-constexpr int xfwd_min_blocks() { return sizeof(R) == 4 && M <= 192 ? 6 : 1; }
+constexpr int xfwd_min_blocks() { return sizeof(R) == 4 && M <= 192 && fft::FourStep<M, kThreads>::N2 <= 16 ? 6 : 1; }
 
 template <class R, int M, class QT, bool kTab = false>
 __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT* __restrict__ src, const double* __restrict__ scale_row,
@@ -469,7 +454,7 @@ __device__ __noinline__ void zfwd_tile(cplx<R>* __restrict__ S, int ny, int nxh,
 }
 
 template <class R, int NZ, bool kTab = false>
-__global__ void __launch_bounds__(kThreads, 4) k_zfwd4(cplx<R>* __restrict__ S, int ny, int nxh,
+__global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, NZ>())) k_zfwd4(cplx<R>* __restrict__ S, int ny, int nxh,
                                                     const cplx<R>* __restrict__ tw_g,
                                                     const FastTab<R>* __restrict__ tab) {
     pdl_wait();
@@ -525,7 +510,7 @@ __device__ __noinline__ void zinv_tile_phi(const cplx<R>* __restrict__ S, cplx<R
 }
 
 template <class R, int NZ, bool kTab = false>
-__global__ void __launch_bounds__(kThreads, 4) k_zinv4(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F,
+__global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, NZ>())) k_zinv4(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F,
                                                     int ny, int nxh, size_t fstride, const double* __restrict__ sinz,
                                                     const cplx<R>* __restrict__ tw_g, int phi_only,
                                                     const FastTab<R>* __restrict__ tab) {
@@ -566,7 +551,7 @@ __device__ __forceinline__ void store_pair(R* p, R a, R b) {
 }
 
 template <class R, int M, bool kTab = false>
-__global__ void __launch_bounds__(kThreads, 4) k_xinv4(const cplx<R>* __restrict__ F, R* __restrict__ E,
+__global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(const cplx<R>* __restrict__ F, R* __restrict__ E,
                                                     double* __restrict__ phi, int ny, int nz, size_t fstride,
                                                     const double* __restrict__ sinx,
                                                     const cplx<R>* __restrict__ tw_g, int want_phi, int want_e,
@@ -689,17 +674,14 @@ int wave_blocks(K kernel, size_t smem, int num_sms, int64_t tiles, int* cache) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)*cache * num_sms));
 }
 
-#define TRIBO_FAST_SIZES(X) X(2) X(3) X(4) X(6) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(384) X(512)
-
-bool fast_len(int n) {
-    switch (n) {
-#define CASE(N) case N:
-        TRIBO_FAST_SIZES(CASE)
-#undef CASE
-        return true;
-        default: return false;
-    }
-}
+// every half length M = nx/2 and length nz of a supported grid: 2^a 3^b, nx and nz up to 1024
+#define TRIBO_X_SIZES(X) \
+    X(2) X(3) X(4) X(6) X(8) X(9) X(12) X(16) X(18) X(24) X(27) X(32) X(36) X(48) X(54) X(64) X(72) X(81) X(96) \
+    X(108) X(128) X(144) X(162) X(192) X(216) X(243) X(256) X(288) X(324) X(384) X(432) X(486) X(512)
+#define TRIBO_Z_SIZES(X) \
+    X(4) X(6) X(8) X(9) X(12) X(16) X(18) X(24) X(27) X(32) X(36) X(48) X(54) X(64) X(72) X(81) X(96) \
+    X(108) X(128) X(144) X(162) X(192) X(216) X(243) X(256) X(288) X(324) X(384) X(432) X(486) X(512) \
+    X(576) X(648) X(729) X(768) X(864) X(972) X(1024)
 
 }  // namespace
 }  // namespace tribo

@@ -52,15 +52,6 @@ template <class R> struct vec4 { R x, y, z, w; };
 template <> struct __align__(16) vec4<float> { float x, y, z, w; };
 template <> struct __align__(32) vec4<double> { double x, y, z, w; };
 
-// ------------------------------------------------------------------ FFT plan
-// Mixed-radix (4, 2, 3) Stockham plan for one transform length.
-struct FftPlan {
-    int n = 0;
-    int npass = 0;
-    int radix[24];
-    void* tw = nullptr;      // device table, n entries of cplx<R>: exp(-2 pi i e / n)
-};
-
 // ------------------------------------------------------------------ context
 struct Accum {                // device-side statistics accumulators
     double sum_wall;          // total charge received from walls
@@ -125,10 +116,7 @@ struct tribo_ctx {
                                  // adjoint uses the same array between its solves)
     void* S = nullptr;           // (nz, ny, nxh) cplx<real> spectrum
     void* F = nullptr;           // (4, nz, ny+2, nxh) cplx<real> field spectra
-    void* W = nullptr;           // (ny, nz*nxh) cplx<double> Thomas scratch (generic path)
-    tribo::FftPlan plan_x, plan_z;
-    // compile-time-length path (poisson_fast.cu)
-    bool fast = false;
+    // transform and y-solve tables (poisson_fast.cu)
     void* d_ytab = nullptr;      // (ny, (nz/2+1)*nxh) double2: 1/pivot, c' per wavenumber pair
     void* W2 = nullptr;          // (ny, (nz/2+1)*nxh, 2) double2 Thomas scratch
     void* d_twx = nullptr;       // nx twiddles exp(-2 pi i e / nx), then the x transform's inner twiddles by thread
@@ -241,6 +229,51 @@ tribo_status cuda_fail(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return ::tribo::cuda_fail(e_, "kernel launch"); \
     } while (0)
 
+// Channel tables: the split passes also run for a group of channels with the
+// same grid in one launch each (a batch's channels, blockIdx.y = channel): the
+// kTab instantiation of a pass takes its channel's arrays from tab[blockIdx.y]
+// instead of its pointer arguments (a separate instantiation, so that the
+// single-channel passes keep their pointers in the parameter space and their
+// register budgets).
+template <class R>
+struct FastTab {
+    void* src;                  // FP64 cell charge sums (forward x source)
+    const double* scale;        // per-row RHS factor
+    cplx<R>* S;                 // spectrum
+    cplx<R>* F;                 // field spectra (the E_y spectrum at F + fstride)
+    R* E;                       // field lattice
+    const cplx<R>* twx;
+    const cplx<R>* twz;
+    const double* sinx;
+    const double* sinz;
+    const float2* tinv;         // y solve (mixed): 1/pivot, c' (double-single), sub-diagonal, E_y coefficients
+    const float2* tcp;
+    const float2* yads;         // y couplings (twisted solve: a_j, c_j), E_y coefficients, chunk checkpoints
+    const float4* yec;
+    float4* yck;
+};
+
+// What the launch of a transform pass needs besides its arrays.  tab != NULL:
+// the pass runs for the n channels of a group, with the arrays of tab[0..n).
+template <class R>
+struct PassGrid {
+    int nx, ny, nz, nxh, num_sms;
+    cudaStream_t stream;
+    const FastTab<R>* tab = nullptr;
+    int n = 1;
+};
+// x and z passes (poisson_x32.cu, ...): set the shared-memory limits of the
+// instantiations for M = nx/2 (nz), then launch
+template <class R> tribo_status xpass_attr(int m, int optin);
+template <class R> tribo_status zpass_attr(int nz, int optin);
+template <class R> void xfwd_launch(const PassGrid<R>& g, void* src, bool src_f64, const double* scale, bool zero,
+                                    cplx<R>* S, const cplx<R>* twx);
+template <class R> void zfwd_launch(const PassGrid<R>& g, cplx<R>* S, const cplx<R>* twz);
+template <class R> void zinv_launch(const PassGrid<R>& g, const cplx<R>* S, cplx<R>* F, const double* sinz,
+                                    const cplx<R>* twz, bool phi_only);
+template <class R> void xinv_launch(const PassGrid<R>& g, const cplx<R>* F, R* E, double* phi, const double* sinx,
+                                    const cplx<R>* twx);
+
 // Poisson (poisson.cu)
 tribo_status poisson_setup(tribo_ctx* c);
 tribo_status poisson_free(tribo_ctx* c);
@@ -248,13 +281,12 @@ tribo_status poisson_free(tribo_ctx* c);
 // caller's FP64 density) or of the real type (the adjoint's charge adjoint);
 // scale: device ny per-row factor giving the RHS -rho/eps; zero_src: write
 // zeros back into src after reading.  phi may be NULL.  E: (3, nz, ny+2, nx)
-// real (E_x, E_y, E_z), or NULL for the potential alone (phi then non-NULL;
-// the generic-length passes still form the field, into the context's E_lat).
+// real (E_x, E_y, E_z), or NULL for the potential alone (phi then non-NULL).
 tribo_status poisson_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
                            double* phi, void* E);
 
-// groups of mixed-precision channels with one compiled-length grid: every split
-// pass of their solves as one launch over all of them (poisson_fast.cu); the
+// groups of mixed-precision channels with one grid: every split pass of their
+// solves as one launch over all of them (poisson_group.cu); the
 // solve reads each channel's FP64 cell sums, zeroes them and writes its field
 // lattice, on `stream`
 bool poisson_group_ok(const tribo_ctx* c);
@@ -262,12 +294,9 @@ tribo_status poisson_group_create(tribo_ctx* const* chans, int n, void** out);
 tribo_status poisson_group_solve(void* grp, cudaStream_t stream, int64_t* launches);
 void poisson_group_free(void* grp);
 
-// compile-time-length Poisson path (poisson_fast.cu)
-bool poisson_fast_supported(int nx, int nz);
+// set-up and solve (poisson_fast.cu)
 tribo_status poisson_fast_setup(tribo_ctx* c);
 void poisson_fast_free(tribo_ctx* c);
-tribo_status poisson_fast_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
-                                double* phi, void* E);
 
 // particles (particles.cu)
 struct PView {               // device views of one particle ensemble
