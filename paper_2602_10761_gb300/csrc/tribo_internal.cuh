@@ -117,8 +117,8 @@ struct tribo_ctx {
     void* S = nullptr;           // (nz, ny, nxh) cplx<real> spectrum
     void* F = nullptr;           // (4, nz, ny+2, nxh) cplx<real> field spectra
     // transform and y-solve tables (poisson_fast.cu)
-    void* d_ytab = nullptr;      // (ny, (nz/2+1)*nxh) double2: 1/pivot, c' per wavenumber pair
-    void* W2 = nullptr;          // (ny, (nz/2+1)*nxh, 2) double2 Thomas scratch
+    void* d_ytab = nullptr;      // y-solve factors, rows of (nz/2+1)*nxh wavenumber pairs: FP64 ny+1 rows of
+                                 // couplings, ny of inverse pivots; mixed 2 x ny rows of float2
     void* d_twx = nullptr;       // nx twiddles exp(-2 pi i e / nx), then the x transform's inner twiddles by thread
     void* d_twz = nullptr;       // nz twiddles
     void* d_yads = nullptr;      // ny float2: y sub-diagonal in double-single (mixed mode)
