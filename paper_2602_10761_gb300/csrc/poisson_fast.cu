@@ -167,10 +167,18 @@ __global__ void __launch_bounds__(128) k_ysolve64(cplx<double>* __restrict__ S, 
     }
 }
 
-// The factors of k_ysolve64 per (|m_z|, m_x), one thread each
-__global__ void k_ytab64(const double* __restrict__ ycoef, const double* __restrict__ lamx,
-                         const double* __restrict__ lamz, int ny, int nz, int nxh, double* __restrict__ te,
-                         double* __restrict__ ti) {
+__device__ __forceinline__ void put_factor(double* p, double v) { *p = v; }
+__device__ __forceinline__ void put_factor(float2* p, double v) {
+    const float hi = (float)v;
+    *p = make_float2(hi, (float)(v - (double)hi));
+}
+
+// The factors of the twisted elimination per (|m_z|, m_x), one thread each, in FP64; T = double, or
+// float2 for the double-single pairs of the mixed solve
+template <class T>
+__global__ void k_ytab(const double* __restrict__ ycoef, const double* __restrict__ lamx,
+                       const double* __restrict__ lamz, int ny, int nz, int nxh, T* __restrict__ te,
+                       T* __restrict__ ti) {
     const int ni = (nz / 2 + 1) * nxh;
     const int item = blockIdx.x * blockDim.x + threadIdx.x;
     if (item >= ni) return;
@@ -178,8 +186,8 @@ __global__ void k_ytab64(const double* __restrict__ ycoef, const double* __restr
     const double *a = ycoef, *b = ycoef + ny, *c = ycoef + 2 * ny;
     const int k = ny >> 1;
     auto put = [&](int j, double e, double i) {
-        te[(size_t)j * ni + item] = e;
-        ti[(size_t)j * ni + item] = i;
+        put_factor(te + (size_t)j * ni + item, e);
+        put_factor(ti + (size_t)j * ni + item, i);
     };
     double up = 0.0, dn = 0.0;
     for (int j = 0; j < k; ++j) {
@@ -194,7 +202,7 @@ __global__ void k_ytab64(const double* __restrict__ ycoef, const double* __restr
     }
     const double e = a[k] * up, f = c[k] * dn;
     put(k, e, 1.0 / ((b[k] - lam) - (k > 0 ? e * c[k - 1] : 0.0) - (k < ny - 1 ? f * a[k + 1] : 0.0)));
-    te[(size_t)ny * ni + item] = f;
+    put_factor(te + (size_t)ny * ni + item, f);
 }
 
 // ---------------------------------------------------------------- fused inverse pipeline
@@ -663,20 +671,12 @@ tribo_status solve_fast(tribo_ctx* c, void* src, bool src_f64, const double* sca
                          (cplx<double>*)c->F + fstride, te, te + (size_t)(ny + 1) * ni, (const double*)c->d_ycoef,
                          (const double*)c->d_ey, ny, nz, nxh, E != nullptr ? 1 : 0);
     } else {
-        const float2* tinv = (const float2*)c->d_ytab;
-        const float2* tcp = tinv + (size_t)ny * ni;
         // without E (the adjoint's potential-only solves) the E_y spectrum is not written
-        // fewer pencils than one 128-thread block per SM (e.g. 128^3: 65 blocks): two threads per
-        // pencil, one half each, meeting through warp shuffles (54 -> 37 us at 128^3, chunks of 8
-        // rows; 5 and 12 rows: 43 and 39 us); otherwise one thread runs both halves
-        const int64_t np = (int64_t)nz * nxh;
-        const bool split = np < 128 * (int64_t)c->num_sms;
-        const int64_t nblk = ((split ? 2 : 1) * np + 127) / 128;
-        auto* ys = split ? (E ? k_ysolve_twist<kTwistC2, true, false, 2> : k_ysolve_twist<kTwistC2, false, false, 2>)
-                         : (E ? k_ysolve_twist<kTwistC> : k_ysolve_twist<kTwistC, false>);
-        (void)launch_pdl(ys, dim3((unsigned)nblk), dim3(128), ysolve_twist_smem(ny), c->stream, (cplx<float>*)c->S,
-                         (cplx<float>*)c->F + fstride, tinv, tcp, (const float2*)c->d_yads,
-                         (const float4*)c->d_yec, (float4*)c->d_yck, ny, nz, nxh, (const FastTab<float>*)nullptr);
+        const float2* te = (const float2*)c->d_ytab;
+        auto solve = E ? ysolve_twist_launch<true, false> : ysolve_twist_launch<false, false>;
+        solve((int64_t)nz * nxh, 1, c->num_sms, ny, c->stream, (cplx<float>*)c->S, (cplx<float>*)c->F, te,
+              te + (size_t)(ny + 1) * ni, (const float2*)c->d_ycpl, (const float4*)c->d_yec, (float4*)c->d_yck, nz, nxh,
+              nullptr);
     }
     TRIBO_LAUNCHED(c);
     if (fused) {
@@ -703,17 +703,7 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
     const std::vector<double>& yf = c->yf;
     const std::vector<double>& yc = c->yc;
     const std::vector<double>& dy = c->dy;
-    // factor table: per (|m_z|, m_x) and row j, (1/pivot_j, c'_j) of the
-    // shifted y operator, in FP64
-    std::vector<double> lamx(nxh), lamz(nz / 2 + 1);
-    for (int m = 0; m < nxh; ++m) {
-        const double s = std::sin(M_PI * m / nx);
-        lamx[m] = 4.0 / (c->dx * c->dx) * s * s;
-    }
-    for (int m = 0; m <= nz / 2; ++m) {
-        const double s = std::sin(M_PI * m / nz);
-        lamz[m] = 4.0 / (c->dz * c->dz) * s * s;
-    }
+    // the y operator, for the couplings and E_y coefficients of the mixed solve
     std::vector<double> a(ny, 0.0), b(ny), cc(ny, 0.0);
     for (int j = 0; j < ny; ++j) {
         if (j >= 1) a[j] = 1.0 / (dy[j] * (yc[j] - yc[j - 1]));
@@ -723,52 +713,24 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
     b[0] -= 1.0 / (dy[0] * (yc[0] - yf[0]));
     b[ny - 1] -= 1.0 / (dy[ny - 1] * (yf[ny] - yc[ny - 1]));
     const bool ds_mode = c->prec != TRIBO_FP64;
-    std::vector<float2> tab32;
-    if (ds_mode) tab32.resize(2 * (size_t)ny * ni);
     const int kmid = ny / 2;         // the twisted solve's middle row
-    for (int item = 0; item < ni && ds_mode; ++item) {
-        const double lam = lamz[item / nxh] + lamx[item % nxh];
-        {
-            // twisted factors: forward (1/pivot_j, c'_j) for rows 0..k-1, backward (1/pivot'_j,
-            // a''_j) for rows ny-1..k+1, and (1/gamma_k, 0) for row k
-            auto put = [&](int j, double u, double v) {
-                float2 t0, t1;
-                split_ds(u, &t0.x, &t0.y);
-                split_ds(v, &t1.x, &t1.y);
-                tab32[(size_t)j * ni + item] = t0;
-                tab32[(size_t)ny * ni + (size_t)j * ni + item] = t1;
-            };
-            double cp = 0.0;
-            for (int j = 0; j < kmid; ++j) {
-                const double inv = 1.0 / ((b[j] - lam) - a[j] * cp);
-                cp = cc[j] * inv;
-                put(j, inv, cp);
-            }
-            double ap = 0.0;
-            for (int j = ny - 1; j > kmid; --j) {
-                const double inv = 1.0 / ((b[j] - lam) - cc[j] * ap);
-                ap = a[j] * inv;
-                put(j, inv, ap);
-            }
-            put(kmid, 1.0 / ((b[kmid] - lam) - a[kmid] * cp - cc[kmid] * ap), 0.0);
-        }
-    }
-    const size_t tab_bytes = 16 * (size_t)ny * ni + 8 * (size_t)ni;
-    TRIBO_CUDA(cudaMalloc(&c->d_ytab, tab_bytes));
+    const size_t rows = 2 * (size_t)ny + 1;
+    TRIBO_CUDA(cudaMalloc(&c->d_ytab, 8 * rows * ni));
     if (ds_mode) {
-        TRIBO_CUDA(cudaMemcpy(c->d_ytab, tab32.data(), sizeof(float2) * tab32.size(), cudaMemcpyHostToDevice));
+        float2* te = (float2*)c->d_ytab;
+        k_ytab<<<(ni + 127) / 128, 128>>>(c->d_ycoef, c->d_lamx, c->d_lamz, ny, nz, nxh, te,
+                                          te + (size_t)(ny + 1) * ni);
     } else {
         double* te = (double*)c->d_ytab;
-        k_ytab64<<<(ni + 127) / 128, 128>>>(c->d_ycoef, c->d_lamx, c->d_lamz, ny, nz, nxh, te,
-                                            te + (size_t)(ny + 1) * ni);
-        TRIBO_CUDA(cudaGetLastError());
+        k_ytab<<<(ni + 127) / 128, 128>>>(c->d_ycoef, c->d_lamx, c->d_lamz, ny, nz, nxh, te,
+                                          te + (size_t)(ny + 1) * ni);
     }
+    TRIBO_CUDA(cudaGetLastError());
     if (ds_mode) {
-        // couplings of the twisted sweeps in double-single: a_j (rows 0..k), c_j (rows k+1..ny-1),
-        // c_k at ny; E_y coefficients per cell and walls
-        std::vector<float2> ads(ny + 1);
-        for (int j = 0; j < ny; ++j) split_ds(j <= kmid ? a[j] : cc[j], &ads[j].x, &ads[j].y);
-        split_ds(cc[kmid], &ads[ny].x, &ads[ny].y);
+        // couplings of the substitution in double-single: c_j (rows 0..k-1), a_j (rows k..ny-1);
+        // E_y coefficients per cell and walls
+        std::vector<float2> cpl(ny);
+        for (int j = 0; j < ny; ++j) split_ds(j < kmid ? cc[j] : a[j], &cpl[j].x, &cpl[j].y);
         auto w = [&](int f) { return (yf[f] - yc[f - 1]) / (yc[f] - yc[f - 1]); };
         std::vector<float4> ec(ny + 1, make_float4(0, 0, 0, 0));
         for (int j = 0; j < ny; ++j) {
@@ -780,10 +742,10 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
             ec[j] = make_float4((float)A, (float)Bm, (float)Bp, 0.f);
         }
         ec[ny] = make_float4((float)(-1.0 / (yc[0] - yf[0])), (float)(1.0 / (yf[ny] - yc[ny - 1])), 0.f, 0.f);
-        TRIBO_CUDA(cudaMalloc(&c->d_yads, sizeof(float2) * (ny + 1)));
-        TRIBO_CUDA(cudaMemcpy(c->d_yads, ads.data(), sizeof(float2) * (ny + 1), cudaMemcpyHostToDevice));
+        TRIBO_CUDA(cudaMalloc(&c->d_ycpl, sizeof(float2) * ny));
+        TRIBO_CUDA(cudaMemcpy(c->d_ycpl, cpl.data(), sizeof(float2) * ny, cudaMemcpyHostToDevice));
         // chunk checkpoints of the twisted sweeps
-        const int cmin = std::min(kTwistC, kTwistC2);        // the launch with more chunks
+        const int cmin = std::min(kTwistC1, kTwistC2);        // the launch with more chunks
         const size_t nck = (size_t)std::max(1, (kmid + cmin - 1) / cmin - 1) * 2 * (size_t)nz * nxh;
         TRIBO_CUDA(cudaMalloc(&c->d_yck, sizeof(float4) * nck));
         TRIBO_CUDA(cudaMalloc(&c->d_yec, sizeof(float4) * (ny + 1)));
@@ -814,17 +776,6 @@ tribo_status poisson_fast_setup(tribo_ctx* c) {
         return xpass_attr<double>(nx / 2, optin);
     }
     if ((st = twiddles<float>(nx, &c->d_twx, true)) || (st = twiddles<float>(nz, &c->d_twz))) return st;
-    if (ysolve_twist_smem(ny) > (size_t)optin) {
-        set_last_error("grid needs more shared memory per block than the device offers");
-        return TRIBO_ERR_UNSUPPORTED;
-    }
-    TRIBO_CUDA(cudaFuncSetAttribute(k_ysolve_twist<kTwistC>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_ysolve_twist<kTwistC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    optin));
-    TRIBO_CUDA(cudaFuncSetAttribute((k_ysolve_twist<kTwistC2, true, false, 2>),
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
-    TRIBO_CUDA(cudaFuncSetAttribute((k_ysolve_twist<kTwistC2, false, false, 2>),
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, optin));
     c->smem_optin = optin;
     if ((st = zpass_attr<float>(nz, optin))) return st;
     return xpass_attr<float>(nx / 2, optin);
@@ -834,13 +785,13 @@ void poisson_fast_free(tribo_ctx* c) {
     cudaFree(c->d_ytab);
     cudaFree(c->d_twx);
     cudaFree(c->d_twz);
-    cudaFree(c->d_yads);
+    cudaFree(c->d_ycpl);
     cudaFree(c->d_yec);
     cudaFree(c->d_yck);
     c->d_yck = nullptr;
     cudaFree(c->ring);
     cudaFree(c->d_pipe);
-    c->d_ytab = c->d_twx = c->d_twz = c->d_yads = c->d_yec = c->ring = c->d_pipe = nullptr;
+    c->d_ytab = c->d_twx = c->d_twz = c->d_ycpl = c->d_yec = c->ring = c->d_pipe = nullptr;
 }
 
 tribo_status poisson_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,

@@ -19,18 +19,9 @@ struct Group {
     FastTab<float>* d_tab = nullptr;
 };
 
-void group_ysolve(const Group& g, cudaStream_t st) {
-    const int64_t nblk = ((int64_t)g.nz * g.nxh + 127) / 128;
-    k_ysolve_twist<kTwistC, true, true><<<dim3((unsigned)nblk, g.n), 128, ysolve_twist_smem(g.ny), st>>>(
-        nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, g.ny, g.nz, g.nxh, g.d_tab);
-}
-
 tribo_status group_attr(const Group& g) {
     tribo_status st;
     if ((st = xpass_attr<float>(g.nx / 2, g.smem_optin)) || (st = zpass_attr<float>(g.nz, g.smem_optin))) return st;
-    if (ysolve_twist_smem(g.ny) > (size_t)g.smem_optin) return TRIBO_ERR_UNSUPPORTED;
-    TRIBO_CUDA(cudaFuncSetAttribute((k_ysolve_twist<kTwistC, true, true>),
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, g.smem_optin));
     return TRIBO_OK;
 }
 
@@ -60,9 +51,9 @@ tribo_status poisson_group_create(tribo_ctx* const* chans, int n, void** out) {
         f.twz = (const cplx<float>*)c->d_twz;
         f.sinx = c->d_sinx;
         f.sinz = c->d_sinz;
-        f.tinv = (const float2*)c->d_ytab;
-        f.tcp = f.tinv + (size_t)c->ny * ni;
-        f.yads = (const float2*)c->d_yads;
+        f.te = (const float2*)c->d_ytab;
+        f.ti = f.te + (size_t)(c->ny + 1) * ni;
+        f.cpl = (const float2*)c->d_ycpl;
         f.yec = (const float4*)c->d_yec;
         f.yck = (float4*)c->d_yck;
     }
@@ -94,7 +85,8 @@ tribo_status poisson_group_solve(void* grp, cudaStream_t stream, int64_t* launch
     const PassGrid<float> pg{g->nx, g->ny, g->nz, g->nxh, g->num_sms, stream, g->d_tab, g->n};
     xfwd_launch<float>(pg, nullptr, true, nullptr, true, nullptr, nullptr);
     zfwd_launch<float>(pg, nullptr, nullptr);
-    group_ysolve(*g, stream);
+    ysolve_twist_launch<true, true>((int64_t)g->nz * g->nxh, g->n, g->num_sms, g->ny, stream, nullptr, nullptr, nullptr,
+                                    nullptr, nullptr, nullptr, nullptr, g->nz, g->nxh, g->d_tab);
     zinv_launch<float>(pg, nullptr, nullptr, nullptr, nullptr, false);
     xinv_launch<float>(pg, nullptr, nullptr, nullptr, nullptr, nullptr);
     TRIBO_CUDA(cudaGetLastError());

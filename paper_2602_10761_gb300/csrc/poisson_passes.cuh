@@ -152,24 +152,22 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
 }
 
 // ---------------------------------------------------------------- y solve, double-single steps
-// a r - b c with one normalisation: the two products' high parts are combined
-// by a two-sum and their error terms (each exact to FP32 rounding of an
-// O(u) correction) are added to the low part.
-__device__ __forceinline__ ds ds_fms(ds a, float r, ds b, ds c) {
-    const float h1 = a.hi * r;
-    const float e1 = fmaf(a.lo, r, fmaf(a.hi, r, -h1));
-    const float h2 = b.hi * c.hi;
-    const float e2 = fmaf(b.lo, c.hi, fmaf(b.hi, c.lo, fmaf(b.hi, c.hi, -h2)));
-    ds s = two_sum(h1, -h2);
-    s.lo += e1 - e2;
-    return fast_two_sum(s.hi, s.lo);
-}
-// d - b c in the same way
+// d - b c with one normalisation: the product's error terms (each exact to FP32
+// rounding of an O(u) correction) are added to the low part of the two-sum of
+// the high parts
 __device__ __forceinline__ ds ds_sub_mul(ds d, ds b, ds c) {
     const float h = b.hi * c.hi;
     const float e = fmaf(b.lo, c.hi, fmaf(b.hi, c.lo, fmaf(b.hi, c.hi, -h)));
     ds s = two_sum(d.hi, -h);
     s.lo += d.lo - e;
+    return fast_two_sum(s.hi, s.lo);
+}
+// the same for an FP32 r
+__device__ __forceinline__ ds ds_sub_mul(float r, ds b, ds c) {
+    const float h = b.hi * c.hi;
+    const float e = fmaf(b.lo, c.hi, fmaf(b.hi, c.lo, fmaf(b.hi, c.hi, -h)));
+    ds s = two_sum(r, -h);
+    s.lo -= e;
     return fast_two_sum(s.hi, s.lo);
 }
 // a - b rounded to FP32: the high parts' difference is exact when they are
@@ -178,263 +176,297 @@ __device__ __forceinline__ ds ds_sub_mul(ds d, ds b, ds c) {
 __device__ __forceinline__ float ds_diff_f(ds a, ds b) { return (a.hi - b.hi) + (a.lo - b.lo); }
 
 // ---------------------------------------------------------------- y solve, twisted (two-ended) Thomas
-// One thread per pencil (m_z, m_x); the factors are those of |m_z|.  The
-// elimination runs from both walls towards the middle row k = ny/2 at once (a twisted
-// factorisation): the top half (rows 0..k-1) eliminates downwards with the
-// forward factors 1/pivot_j, c'_j = c_j/pivot_j, the bottom half (rows
-// ny-1..k+1) upwards with the backward factors 1/pivot'_j, a''_j =
-// a_j/pivot'_j, and row k joins them with 1/gamma_k, gamma_k = b_k - lam -
-// a_k c'_k-1 - c_k a''_k+1 (all FP64-computed at set-up, one table row per
-// (|m_z|, m_x)).  The two halves are independent chains of half the length,
-// interleaved in one thread: four double-single recurrences (real and
-// imaginary part of each half) instead of two.  In local index t of a half
-// (t = j in the top half, t = ny-1-j in the bottom half) both halves run the
-// same recurrences: p_t = (1/pivot)(r - coupling p_t-1), coupling = a_j
-// (top) or c_j (bottom), and x_t = p_t - (c' or a'') x_t+1 with x at local
-// index H (the half's length) = x_k.  The forward sweep keeps only the value
-// entering each chunk of C rows (in global memory, where they stay in L2),
-// and the substitution walks the chunks back from the middle, recomputing
-// each chunk's forward values into registers from its checkpoint.  E_y per cell j is A_j x_j + Bm_j (x_j - x_j-1) + Bp_j (x_j+1 -
-// x_j) from the double-single values, one cell behind the substitution (the
-// bottom half, walking j upwards, takes Bm and Bp with their roles and signs
+// The elimination runs from both walls towards the middle row k = ny/2 at once
+// (a twisted factorisation): the top half (rows 0..k-1) downwards, the bottom
+// half (rows ny-1..k+1) upwards.  With the pivots' inverses i_j, FP64-computed
+// at set-up per (|m_z|, m_x) and held as double-single pairs:
+//   top     P_j = r_j - e_j P_j-1,  e_j = a_j i_j-1,  x_j = i_j (P_j - c_j x_j+1)
+//   bottom  P_j = r_j - f_j P_j+1,  f_j = c_j i_j+1,  x_j = i_j (P_j - a_j x_j-1)
+//   middle  x_k = g (r_k - e_k P_k-1 - f_k P_k+1).
+// In local index t of a half (t = j in the top half, ny-1-j in the bottom half)
+// both halves run the same recurrences.  E_y per cell j is A_j x_j + Bm_j (x_j -
+// x_j-1) + Bp_j (x_j+1 - x_j) from the double-single values, one cell behind the
+// substitution (the bottom half takes Bm and Bp with their roles and signs
 // exchanged); the top half writes cell k; wall nodes E_y = ew0 phi_0 (bottom
 // wall), ewN phi_ny-1 (top wall).
-// coup: ny + 1 double-single couplings, a_j (j <= k), c_j (j > k), c_k at ny.
+//
+// The forward sweep keeps the value entering each chunk of C rows and the
+// substitution recomputes each chunk's values from it (keeping all of them
+// instead measured the same on small grids and 20 us more at 384x256x256).  A
+// row's values are fetched C rows ahead, into the registers the row C before it
+// has just left, and rows are addressed by 32-bit element indices: the kernel is
+// bound by its instruction stream and its loads' latency together (51% issue,
+// 34% of stalls on loads before this form).  NH = 1: a pencil's halves run in two
+// lanes 16 apart and meet through shuffles; NH = 2: one thread runs both, two
+// interleaved chains.
+// Which one: NH = 1 needs 128 registers for C = 6 rows ahead, four blocks of 64
+// pencils a SM; while the grid fits one such wave it is the faster (us, against
+// 64-pencil blocks of NH = 2, C = 5 at 168 registers): 128^3 24 / 32, 192x128x128
+// 26 / 32, 288x145x162 38 / 53, 256^3 85 / 105; past it (384x256x256, 1.27
+// waves) 153 / 127.  Before: 33 at 128^3, 65 at 288x145x162, 150 at 384x256x256.
+// te: e_j (j <= k) and f_j (j > k), f_k at row ny; ti: i_j, g at row k.
+// cpl: ny couplings c_j (j < k), a_j (j > k).
 // ck: (ceil(k / C) - 1) x 2 x (nz nxh) float4 of chunk checkpoints.
-#ifndef TRIBO_TWIST_C
-#define TRIBO_TWIST_C 5
-#endif
-constexpr int kTwistC = TRIBO_TWIST_C;       // rows per chunk of the twisted solve
-#ifndef TRIBO_TWIST_C2
-#define TRIBO_TWIST_C2 8
-#endif
-constexpr int kTwistC2 = TRIBO_TWIST_C2;     // ... with two threads per pencil
-// shared memory of a twisted solve: E_y coefficients and couplings, ny + 1 each
-inline size_t ysolve_twist_smem(int ny) { return (sizeof(float4) + sizeof(float2)) * (size_t)(ny + 1); }
+constexpr int kTwistC1 = 6, kTwistT1 = 128;  // NH = 1: rows per chunk, threads per block
+constexpr int kTwistC2 = 5, kTwistT2 = 64;   // NH = 2
+// shared memory: the E_y coefficients of both halves and the couplings
+inline size_t ysolve_twist_smem(int ny) { return (2 * sizeof(float4) + sizeof(float2)) * (size_t)(ny + 1); }
+// the pencils of one resident wave of the NH = 1 form
+inline bool ysolve_two_lanes(int64_t pencils, int num_sms) { return pencils <= (int64_t)num_sms * 4 * (kTwistT1 / 2); }
 
-// SPLIT = 1: one thread runs both halves of its pencil (many pencils); SPLIT = 2: two adjacent
-// threads run one half each and meet through warp shuffles (few pencils, where a thread's
-// instruction stream, not the number of warps, sets the time).
-template <int C, bool EY = true, bool kTab = false, int SPLIT = 1>
-__global__ void __launch_bounds__(128, 3) k_ysolve_twist(cplx<float>* __restrict__ S, cplx<float>* __restrict__ Fy,
-                                                         const float2* __restrict__ tinv,
-                                                         const float2* __restrict__ tcp,
-                                                         const float2* __restrict__ coup,
-                                                         const float4* __restrict__ ec, float4* __restrict__ ck,
-                                                         int ny, int nz, int nxh,
-                                                         const FastTab<float>* __restrict__ tab) {
+template <int NH, bool EY = true, bool kTab = false>
+__global__ void __launch_bounds__(NH == 1 ? kTwistT1 : kTwistT2, NH == 1 ? 4 : 6)
+k_ysolve_twist(cplx<float>* __restrict__ S, cplx<float>* __restrict__ F, const float2* __restrict__ te,
+               const float2* __restrict__ ti, const float2* __restrict__ cpl, const float4* __restrict__ ec,
+               float4* __restrict__ ck, int ny, int nz, int nxh, const FastTab<float>* __restrict__ tab) {
+    constexpr int C = NH == 1 ? kTwistC1 : kTwistC2;
     pdl_wait();
     if constexpr (kTab) {
         const FastTab<float>& t = tab[blockIdx.y];
         S = t.S;
-        Fy = t.F + (size_t)nz * (ny + 2) * nxh;
-        tinv = t.tinv;
-        tcp = t.tcp;
-        coup = t.yads;
+        F = t.F;
+        te = t.te;
+        ti = t.ti;
+        cpl = t.cpl;
         ec = t.yec;
         ck = t.yck;
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float4* se = reinterpret_cast<float4*>(smem_raw);                 // ny + 1
-    float2* sa = reinterpret_cast<float2*>(se + ny + 1);              // ny + 1
+    float4* se = reinterpret_cast<float4*>(smem_raw);                 // 2 x (ny + 1): top, bottom
+    float2* sc = reinterpret_cast<float2*>(se + 2 * (ny + 1));        // ny
     for (int j = threadIdx.x; j <= ny; j += blockDim.x) {
-        sa[j] = coup[j];
-        se[j] = ec[j];
+        if (j < ny) sc[j] = cpl[j];
+        const float4 c = ec[j];
+        se[j] = c;
+        se[ny + 1 + j] = make_float4(c.x, -c.z, -c.y, 0.f);
     }
     __syncthreads();
-    constexpr int NH = SPLIT == 2 ? 1 : 2;                            // halves per thread
-    const int np = nz * nxh;
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int pencil = SPLIT == 2 ? gtid >> 1 : gtid;
-    const int h0 = SPLIT == 2 ? (gtid & 1) : 0;                        // this thread's first half
-    // the two threads of a pencil are both in or both out
-    const unsigned live = SPLIT == 2 ? __ballot_sync(0xffffffffu, pencil < np) : 0u;
-    if (pencil >= np) return;
-    const int ni = (nz / 2 + 1) * nxh;
-    const int mz = pencil / nxh;
-    const int mx = pencil - mz * nxh;
-    const int item = min(mz, nz - mz) * nxh + mx;
-    cplx<float>* srow = S + (size_t)mz * ny * nxh + mx;
-    cplx<float>* frow = Fy + (size_t)mz * (ny + 2) * nxh + mx;
+    constexpr int PW = NH == 1 ? 16 : 32;                             // pencils per warp
+    const int lane = threadIdx.x & 31;
+    const int h0 = NH == 1 ? (lane >> 4) : 0;                         // this thread's first half
+    const uint32_t np = (uint32_t)nz * nxh, ni = (uint32_t)(nz / 2 + 1) * nxh;
+    const uint32_t pencil = (blockIdx.x * blockDim.x + threadIdx.x) / 32 * PW + lane % PW;
+    const bool live = pencil < np;
+    if (NH == 2 && !live) return;
+    const uint32_t mz = live ? pencil / nxh : 0, mx = live ? pencil - mz * nxh : 0;
+    const uint32_t item = min(mz, (uint32_t)nz - mz) * nxh + mx;
     const int k = ny >> 1;
-    const int hl[2] = {k, ny - 1 - k};            // rows of the top and the bottom half
-    const int nch = (k + C - 1) / C;
-    // forward elimination of the thread's halves, checkpoints at the end of each chunk but the last
-    ds p[NH][2];
+    // element indices of row 0 (a grid of at most 1024 cells a side has fewer than 2^32 elements)
+    float2* const Sv = reinterpret_cast<float2*>(S);
+    float2* const Yv = reinterpret_cast<float2*>(F + (size_t)nz * (ny + 2) * nxh);   // E_y spectrum
+    const uint32_t rs = nxh;
+    const uint32_t s0 = mz * ny * nxh + mx, f0 = mz * (ny + 2) * nxh + mx;
+    auto pair = [](float2 v) { return ds{v.x, v.y}; };
+    // per half of the thread: rows, row of local row 0 and its direction
+    int H[NH], Hmin = 1 << 30, j0[NH];
+    uint32_t d[NH];                                                   // +1, -1 (modulo 2^32)
 #pragma unroll
-    for (int hh = 0; hh < NH; ++hh) p[hh][0] = p[hh][1] = ds{0.f, 0.f};
-    for (int c = 0; c < nch; ++c) {
-        float2 tv[NH][C];
-        cplx<float> rv[NH][C];
+    for (int hh = 0; hh < NH; ++hh) {
+        const int h = h0 + hh;
+        H[hh] = !live ? 0 : h == 0 ? k : ny - 1 - k;
+        j0[hh] = h == 0 ? 0 : ny - 1;
+        d[hh] = h == 0 ? 1u : ~0u;
+        Hmin = min(Hmin, H[hh]);
+    }
+    // element index of local row t
+    auto at = [&](uint32_t base, uint32_t stride, int hh, int t) {
+        return base + ((uint32_t)j0[hh] + d[hh] * (uint32_t)t) * stride;
+    };
+    const int nch = live ? (k + C - 1) / C : 0;                       // the top half is the longer one
+    // ---- forward elimination
+    ds P[NH][2];
+    float2 e[NH][C], r[NH][C];
 #pragma unroll
-        for (int hh = 0; hh < NH; ++hh)
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const int h = h0 + hh, t = c * C + i;
-                if (t < hl[h]) {
-                    const int j = h == 0 ? t : ny - 1 - t;
-                    tv[hh][i] = tinv[(size_t)j * ni + item];
-                    rv[hh][i] = srow[(size_t)j * nxh];
-                }
-            }
+    for (int hh = 0; hh < NH; ++hh) {
+        P[hh][0] = P[hh][1] = ds{0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < C; ++i)
-#pragma unroll
-            for (int hh = 0; hh < NH; ++hh) {
-                const int h = h0 + hh, t = c * C + i;
-                if (t < hl[h]) {
-                    const int j = h == 0 ? t : ny - 1 - t;
-                    const ds inv = {tv[hh][i].x, tv[hh][i].y};
-                    const ds at = ds_mul(ds{sa[j].x, sa[j].y}, inv);
-                    p[hh][0] = ds_fms(inv, rv[hh][i].re, at, p[hh][0]);
-                    p[hh][1] = ds_fms(inv, rv[hh][i].im, at, p[hh][1]);
-                }
+            if (i < H[hh]) {
+                e[hh][i] = te[at(item, ni, hh, i)];
+                r[hh][i] = Sv[at(s0, rs, hh, i)];
             }
+    }
+    for (int c = 0; c < nch; ++c) {
+        const int t0 = c * C;
+        auto rows = [&](auto full) {          // full: every row of the chunk lies in both halves
+#pragma unroll
+            for (int i = 0; i < C; ++i)
+#pragma unroll
+                for (int hh = 0; hh < NH; ++hh)
+                    if (decltype(full)::value || t0 + i < H[hh]) {
+                        P[hh][0] = ds_sub_mul(r[hh][i].x, pair(e[hh][i]), P[hh][0]);
+                        P[hh][1] = ds_sub_mul(r[hh][i].y, pair(e[hh][i]), P[hh][1]);
+                        if (t0 + i + C < H[hh]) {
+                            e[hh][i] = te[at(item, ni, hh, t0 + i + C)];
+                            r[hh][i] = Sv[at(s0, rs, hh, t0 + i + C)];
+                        }
+                    }
+        };
+        if (t0 + C <= Hmin) rows(std::true_type{});
+        else rows(std::false_type{});
         if (c + 1 < nch)
 #pragma unroll
             for (int hh = 0; hh < NH; ++hh)
                 ck[((size_t)c * 2 + h0 + hh) * np + pencil] =
-                    make_float4(p[hh][0].hi, p[hh][0].lo, p[hh][1].hi, p[hh][1].lo);
+                    make_float4(P[hh][0].hi, P[hh][0].lo, P[hh][1].hi, P[hh][1].lo);
     }
-    // both halves' last forward values (the other thread's through a shuffle)
-    ds pa[2][2];
-    if constexpr (SPLIT == 2) {
+    // ---- the middle row (the other half's last forward value through a shuffle when another
+    // thread has it), and each half's row next to it
+    auto other = [&](ds v) {
+        return ds{__shfl_xor_sync(0xffffffffu, v.hi, 16), __shfl_xor_sync(0xffffffffu, v.lo, 16)};
+    };
+    ds xk[2], xn[NH][2], x1[NH][2];          // x1: x at local row t + 1
+    float dn[NH][2];                         // x(t + 2) - x(t + 1), zero where the other half is empty
+    {
+        ds po[2];                            // the forward value of the first half's other half
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
-            pa[h0][m] = p[0][m];
-            pa[1 - h0][m] = ds{__shfl_xor_sync(live, p[0][m].hi, 1), __shfl_xor_sync(live, p[0][m].lo, 1)};
+            if constexpr (NH == 2) po[m] = P[1][m];
+            else po[m] = other(P[0][m]);
+            xk[m] = xn[0][m] = ds{0.f, 0.f};
         }
-    } else {
+        if (live) {
+            const ds ek = pair(te[item + (uint32_t)k * ni]), fk = pair(te[item + (uint32_t)ny * ni]);
+            const ds g = pair(ti[item + (uint32_t)k * ni]);
+            const float2 rk = Sv[s0 + (uint32_t)k * rs];
 #pragma unroll
-        for (int m = 0; m < 2; ++m) {
-            pa[0][m] = p[0][m];
-            pa[1][m] = p[NH - 1][m];
-        }
-    }
-    // the middle row: x_k = (r_k - a_k d_k-1 - c_k e_k+1) / gamma_k (d, e zero for an empty half)
-    const float2 tk = tinv[(size_t)k * ni + item];
-    const ds ig = {tk.x, tk.y};
-    const cplx<float> rk = srow[(size_t)k * nxh];
-    const ds ga = ds_mul(ig, ds{sa[k].x, sa[k].y});
-    const ds gc = ds_mul(ig, ds{sa[ny].x, sa[ny].y});
-    ds xk[2];
-    xk[0] = ds_sub_mul(ds_fms(ig, rk.re, ga, pa[0][0]), gc, pa[1][0]);
-    xk[1] = ds_sub_mul(ds_fms(ig, rk.im, ga, pa[0][1]), gc, pa[1][1]);
-    if (h0 == 0) srow[(size_t)k * nxh] = cplx<float>{ds_f(xk[0]), ds_f(xk[1])};
-    // each half's row next to k (x_k-1, x_k+1): the start of the other half's E_y differences
-    ds xn[2][2];
+            for (int m = 0; m < 2; ++m) {
+                const ds pt = h0 == 0 ? P[0][m] : po[m], pb = h0 == 0 ? po[m] : P[0][m];
+                xk[m] = ds_mul(ds_sub_mul(ds_sub_mul(m ? rk.y : rk.x, ek, pt), fk, pb), g);
+            }
+            if (h0 == 0) Sv[s0 + (uint32_t)k * rs] = make_float2(ds_f(xk[0]), ds_f(xk[1]));
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        xn[h][0] = xk[0];
-        xn[h][1] = xk[1];
-        if (hl[h] > 0) {
-            const int j = h == 0 ? k - 1 : k + 1;
-            const float2 cv = tcp[(size_t)j * ni + item];
-            const ds cp = {cv.x, cv.y};
-            xn[h][0] = ds_sub_mul(pa[h][0], cp, xk[0]);
-            xn[h][1] = ds_sub_mul(pa[h][1], cp, xk[1]);
-        }
-    }
-    ds x1[NH][2];                   // x at local index t + 1
-    float dn[NH][2];                // x(t + 2) - x(t + 1)
+            for (int hh = 0; hh < NH; ++hh) {
+                xn[hh][0] = xk[0];
+                xn[hh][1] = xk[1];
+                if (H[hh] > 0) {
+                    const ds cj = pair(sc[j0[hh] + (int)d[hh] * (H[hh] - 1)]);
+                    const ds iv = pair(ti[at(item, ni, hh, H[hh] - 1)]);
 #pragma unroll
-    for (int hh = 0; hh < NH; ++hh) {
-        const int h = h0 + hh;
-        x1[hh][0] = xk[0];
-        x1[hh][1] = xk[1];
-        const bool other = hl[1 - h] > 0;
-        dn[hh][0] = other ? ds_diff_f(xn[1 - h][0], xk[0]) : 0.f;
-        dn[hh][1] = other ? ds_diff_f(xn[1 - h][1], xk[1]) : 0.f;
-    }
-    // substitution, chunks from the middle outwards, each recomputed from its checkpoint
-    for (int c = nch - 1; c >= 0; --c) {
-        ds q[NH][2];
-#pragma unroll
-        for (int hh = 0; hh < NH; ++hh) {
-            if (c > 0) {
-                const float4 v = ck[((size_t)(c - 1) * 2 + h0 + hh) * np + pencil];
-                q[hh][0] = ds{v.x, v.y};
-                q[hh][1] = ds{v.z, v.w};
-            } else {
-                q[hh][0] = ds{0.f, 0.f};
-                q[hh][1] = ds{0.f, 0.f};
+                    for (int m = 0; m < 2; ++m) xn[hh][m] = ds_mul(ds_sub_mul(P[hh][m], cj, xk[m]), iv);
+                }
             }
         }
-        float2 tv[NH][C], cv[NH][C];
-        cplx<float> rv[NH][C];
+        const int Ho = h0 == 0 ? ny - 1 - k : k;      // rows of the first half's other half
 #pragma unroll
         for (int hh = 0; hh < NH; ++hh)
 #pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const int h = h0 + hh, t = c * C + i;
-                if (t < hl[h]) {
-                    const int j = h == 0 ? t : ny - 1 - t;
-                    tv[hh][i] = tinv[(size_t)j * ni + item];
-                    cv[hh][i] = tcp[(size_t)j * ni + item];
-                    rv[hh][i] = srow[(size_t)j * nxh];
-                }
+            for (int m = 0; m < 2; ++m) {
+                ds xo;
+                if constexpr (NH == 2) xo = xn[1 - hh][m];
+                else xo = other(xn[hh][m]);
+                x1[hh][m] = xk[m];
+                dn[hh][m] = (hh == 0 ? Ho : k) > 0 ? ds_diff_f(xo, xk[m]) : 0.f;
             }
-        ds dr[NH][C], di[NH][C];
+    }
+    if (!live) return;
+    // ---- substitution, chunks from the middle outwards
+    float2 v[NH][C];
+    float4 q[NH];                            // the value entering the chunk
+    int Hs[NH];                              // E_y rows: the bottom half leaves row k to the top
+    const float4* sh[NH];
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh) {
+        Hs[hh] = h0 + hh == 0 ? k + 1 : ny - 1 - k;
+        sh[hh] = se + (h0 + hh) * (ny + 1);
+    }
+    auto fetch = [&](int hh, int i, int t) {
+        v[hh][i] = ti[at(item, ni, hh, t)];
+        r[hh][i] = Sv[at(s0, rs, hh, t)];
+        e[hh][i] = te[at(item, ni, hh, t)];
+    };
+    auto fetch_ck = [&](int c) {
+#pragma unroll
+        for (int hh = 0; hh < NH; ++hh)
+            q[hh] = c > 0 ? ck[((size_t)(c - 1) * 2 + h0 + hh) * np + pencil] : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+#pragma unroll
+    for (int hh = 0; hh < NH; ++hh)
 #pragma unroll
         for (int i = 0; i < C; ++i)
+            if ((nch - 1) * C + i < H[hh]) fetch(hh, i, (nch - 1) * C + i);
+    fetch_ck(nch - 1);
+    for (int c = nch - 1; c >= 0; --c) {
+        const int t0 = c * C;
+        auto rows = [&](auto full) {
+            ds p[NH][C][2], w[NH][2];
 #pragma unroll
             for (int hh = 0; hh < NH; ++hh) {
-                const int h = h0 + hh, t = c * C + i;
-                if (t < hl[h]) {
-                    const int j = h == 0 ? t : ny - 1 - t;
-                    const ds inv = {tv[hh][i].x, tv[hh][i].y};
-                    const ds at = ds_mul(ds{sa[j].x, sa[j].y}, inv);
-                    q[hh][0] = ds_fms(inv, rv[hh][i].re, at, q[hh][0]);
-                    q[hh][1] = ds_fms(inv, rv[hh][i].im, at, q[hh][1]);
-                    dr[hh][i] = q[hh][0];
-                    di[hh][i] = q[hh][1];
-                }
+                w[hh][0] = ds{q[hh].x, q[hh].y};
+                w[hh][1] = ds{q[hh].z, q[hh].w};
             }
 #pragma unroll
-        for (int i = C - 1; i >= 0; --i)
+            for (int i = 0; i < C; ++i)
 #pragma unroll
-            for (int hh = 0; hh < NH; ++hh) {
-                const int h = h0 + hh, t = c * C + i;
-                if (t < hl[h]) {
-                    const int j = h == 0 ? t : ny - 1 - t;
-                    const ds cp = {cv[hh][i].x, cv[hh][i].y};
-                    const ds xr = ds_sub_mul(dr[hh][i], cp, x1[hh][0]);
-                    const ds xi = ds_sub_mul(di[hh][i], cp, x1[hh][1]);
-                    srow[(size_t)j * nxh] = cplx<float>{ds_f(xr), ds_f(xi)};
-                    const float d0r = ds_diff_f(x1[hh][0], xr), d0i = ds_diff_f(x1[hh][1], xi);
-                    // E_y of the cell at local index t + 1 (the bottom half leaves cell k to the top)
-                    if (EY && (h == 0 || t + 1 < hl[1])) {
-                        const int jc = h == 0 ? t + 1 : ny - 2 - t;
-                        const float4 cf = se[jc];
-                        const float bm = h == 0 ? cf.y : -cf.z, bp = h == 0 ? cf.z : -cf.y;
-                        frow[(size_t)(jc + 1) * nxh] = cplx<float>{
-                            cf.x * ds_f(x1[hh][0]) + bm * d0r + bp * dn[hh][0],
-                            cf.x * ds_f(x1[hh][1]) + bm * d0i + bp * dn[hh][1]};
+                for (int hh = 0; hh < NH; ++hh)
+                    if (decltype(full)::value || t0 + i < H[hh]) {
+                        p[hh][i][0] = w[hh][0] = ds_sub_mul(r[hh][i].x, pair(e[hh][i]), w[hh][0]);
+                        p[hh][i][1] = w[hh][1] = ds_sub_mul(r[hh][i].y, pair(e[hh][i]), w[hh][1]);
                     }
-                    dn[hh][0] = d0r;
-                    dn[hh][1] = d0i;
-                    x1[hh][0] = xr;
-                    x1[hh][1] = xi;
-                }
-            }
+            fetch_ck(c - 1);
+#pragma unroll
+            for (int i = C - 1; i >= 0; --i)
+#pragma unroll
+                for (int hh = 0; hh < NH; ++hh)
+                    if (decltype(full)::value || t0 + i < H[hh]) {
+                        const int t = t0 + i, j = j0[hh] + (int)d[hh] * t;
+                        const ds cj = pair(sc[j]), iv = pair(v[hh][i]);
+                        const float4 cf = sh[hh][j + (int)d[hh]];      // coefficients of the row of x1
+                        float xf[2], ey[2];
+#pragma unroll
+                        for (int m = 0; m < 2; ++m) {
+                            const ds x = ds_mul(ds_sub_mul(p[hh][i][m], cj, x1[hh][m]), iv);
+                            xf[m] = ds_f(x);
+                            const float d0 = ds_diff_f(x1[hh][m], x);
+                            ey[m] = cf.x * ds_f(x1[hh][m]) + cf.y * d0 + cf.z * dn[hh][m];
+                            dn[hh][m] = d0;
+                            x1[hh][m] = x;
+                        }
+                        Sv[at(s0, rs, hh, t)] = make_float2(xf[0], xf[1]);
+                        if (EY && t + 1 < Hs[hh]) Yv[at(f0 + rs, rs, hh, t + 1)] = make_float2(ey[0], ey[1]);
+                        if (c > 0) fetch(hh, i, t - C);
+                    }
+        };
+        if (t0 + C <= Hmin) {
+            rows(std::true_type{});
+        } else {
+            rows(std::false_type{});
+            // rows past the end of a half hold nothing to replace: their registers take the next
+            // chunk's values here
+            if (c > 0)
+#pragma unroll
+                for (int hh = 0; hh < NH; ++hh)
+#pragma unroll
+                    for (int i = 0; i < C; ++i)
+                        if (t0 + i >= H[hh]) fetch(hh, i, t0 + i - C);
+        }
     }
     if (!EY) return;
     const float4 walls = se[ny];
 #pragma unroll
     for (int hh = 0; hh < NH; ++hh) {
-        const float xr = ds_f(x1[hh][0]), xi = ds_f(x1[hh][1]);
-        if (h0 + hh == 0) {         // top: cell 0 (node 1) and the wall node 0
-            const float4 cf = se[0];
-            frow[(size_t)1 * nxh] = cplx<float>{cf.x * xr + cf.z * dn[hh][0], cf.x * xi + cf.z * dn[hh][1]};
-            frow[0] = cplx<float>{walls.x * xr, walls.x * xi};
-        } else {                    // bottom: cell ny-1 (node ny) unless it is cell k, and the wall node ny+1
-            if (hl[1] > 0) {
-                const float4 cf = se[ny - 1];
-                frow[(size_t)ny * nxh] = cplx<float>{cf.x * xr - cf.y * dn[hh][0], cf.x * xi - cf.y * dn[hh][1]};
-            }
-            frow[(size_t)(ny + 1) * nxh] = cplx<float>{walls.y * xr, walls.y * xi};
-        }
+        const bool top = h0 + hh == 0;
+        // top: cell 0 (node 1) and the wall node 0; bottom: cell ny-1 (node ny) unless it is cell k,
+        // and the wall node ny+1
+        const float4 cf = sh[hh][top ? 0 : ny - 1];
+        const float x = ds_f(x1[hh][0]), y = ds_f(x1[hh][1]), w = top ? walls.x : walls.y;
+        if (top || H[hh] > 0)
+            Yv[f0 + (uint32_t)(top ? 1 : ny) * rs] = make_float2(cf.x * x + cf.z * dn[hh][0], cf.x * y + cf.z * dn[hh][1]);
+        Yv[f0 + (uint32_t)(top ? 0 : ny + 1) * rs] = make_float2(w * x, w * y);
     }
+}
+
+// launch of the solve for np pencils (n channels): the form by the rule above
+template <bool EY, bool kTab>
+void ysolve_twist_launch(int64_t pencils, int n, int num_sms, int ny, cudaStream_t stream, cplx<float>* S,
+                         cplx<float>* F, const float2* te, const float2* ti, const float2* cpl, const float4* ec,
+                         float4* ck, int nz, int nxh, const FastTab<float>* tab) {
+    const bool two = ysolve_two_lanes(pencils * n, num_sms);
+    const int per = two ? kTwistT1 / 2 : kTwistT2;
+    const dim3 grid((unsigned)((pencils + per - 1) / per), (unsigned)n);
+    (void)launch_pdl(two ? k_ysolve_twist<1, EY, kTab> : k_ysolve_twist<2, EY, kTab>, grid,
+                     dim3(two ? kTwistT1 : kTwistT2), ysolve_twist_smem(ny), stream, S, F, te, ti, cpl, ec, ck, ny, nz,
+                     nxh, tab);
 }
 
 // ---------------------------------------------------------------- z passes (four-step)

@@ -121,7 +121,7 @@ struct tribo_ctx {
                                  // couplings, ny of inverse pivots; mixed 2 x ny rows of float2
     void* d_twx = nullptr;       // nx twiddles exp(-2 pi i e / nx), then the x transform's inner twiddles by thread
     void* d_twz = nullptr;       // nz twiddles
-    void* d_yads = nullptr;      // ny float2: y sub-diagonal in double-single (mixed mode)
+    void* d_ycpl = nullptr;      // ny float2: couplings of the y substitution in double-single (mixed mode)
     void* d_yec = nullptr;       // ny+1 float4: E_y coefficients per cell, walls (mixed mode)
     void* d_yck = nullptr;       // chunk checkpoints of the twisted y sweeps (mixed mode)
     int test_stall_plane = -1;   // testing: a pipelined-inverse plane whose consumers' waits run out
@@ -246,9 +246,9 @@ struct FastTab {
     const cplx<R>* twz;
     const double* sinx;
     const double* sinz;
-    const float2* tinv;         // y solve (mixed): 1/pivot, c' (double-single), sub-diagonal, E_y coefficients
-    const float2* tcp;
-    const float2* yads;         // y couplings (twisted solve: a_j, c_j), E_y coefficients, chunk checkpoints
+    const float2* te;           // y solve (mixed): eliminating couplings and inverse pivots (double-single),
+    const float2* ti;
+    const float2* cpl;          // substitution couplings per row, E_y coefficients, chunk checkpoints
     const float4* yec;
     float4* yck;
 };
