@@ -175,8 +175,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_adj_step(StepArgs<R> a, AdjArgs
                 else tau = tau_p / ((R)1 + rpow23(re) / (R)6);
             }
             s = a.dt / tau;
-            phi1 = -rexpm1(-s);
-            phi2 = phi2_of(s, phi1);
+            if constexpr (sizeof(R) == 8) {
+                phi12(s, phi1, phi2);
+            } else {
+                phi1 = -rexpm1(-s);
+                phi2 = phi2_of(s, phi1);
+            }
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
                 T[c] = uf[c] + acc[c] * tau;

@@ -21,15 +21,20 @@ constexpr int kThreads = 256;
 #define TRIBO_KSTEP_MINB 4
 #endif
 constexpr int kStepThreads = TRIBO_KSTEP_THREADS;
-constexpr int kStepMinBlocks = TRIBO_KSTEP_MINB;
+#ifndef TRIBO_KSTEP_MINB64
+#define TRIBO_KSTEP_MINB64 3
+#endif
+template <class R> constexpr int step_min_blocks() { return sizeof(R) == 4 ? TRIBO_KSTEP_MINB : TRIBO_KSTEP_MINB64; }
 
 template <class R>
 struct StepArgs {
     int nx, ny, nz, nyn;
     R lx, ly, lz, inv_dx, inv_dz, dt;
     R inv_lx, inv_lz;
-    double dx, dz;                 // FP64 cell sizes (exact locate in FP64 mode)
     const double* yf;              // ny+1 FP64 faces
+    const double* xf;              // nx+1 FP64 faces i dx (FP64 mode)
+    const double* zf;              // nz+1
+    float inv_dxf, inv_dzf, ybin_scalef;   // FP32 copies for the FP64 locate's first guess
     const float* yf_up;            // ny+1 rounded-up float faces
     const float* xf_up;            // nx+1
     const float* zf_up;            // nz+1
@@ -80,14 +85,32 @@ template <> __device__ __forceinline__ double rsqrt_<double>(double v) { return 
 template <class R> __device__ __forceinline__ R rpow23(R v);
 template <> __device__ __forceinline__ float rpow23<float>(float v) { return cbrtf(v * v); }
 template <> __device__ __forceinline__ double rpow23<double>(double v) { return cbrt(v * v); }
-template <class R> __device__ __forceinline__ bool rfinite(R v) { return isfinite(v); }
 
-// largest i in [0, n-1] with s >= face_i, faces i*h (FP64) -------------------
-__device__ __forceinline__ int cell_uniform(double s, double h, int n, const float*, double) {
-    int i = (int)floor(s / h);
+// ---- FP64 values on the integer pipes: an FP64 instruction (compares and conversions included)
+// issues at 1/64 of the FP32 rate here, so the locate's first guess is formed in FP32 from the
+// leading bits, and doubles are compared as 64-bit integers, whose order is theirs for
+// non-negative numbers (every face is one; a negative number is below all faces either way)
+__device__ __forceinline__ float lead_f32(double s) {
+    // |s| cut to FP32's 24 bits in its normal range, 0 below it: the exponent and mantissa moved to
+    // their FP32 places, the exponent's bias less by 896
+    const unsigned hi = (unsigned)__double2hiint(s);
+    const unsigned v = __funnelshift_l((unsigned)__double2loint(s), hi, 3) - (896u << 23);
+    return (hi & 0x7fffffffu) < 0x38100000u ? 0.f : __uint_as_float(v);
+}
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+// s as an ordered integer; infinities and NaN below everything
+__device__ __forceinline__ long long order64(double s) { return finite64(s) ? __double_as_longlong(s) : -1ll; }
+__device__ __forceinline__ long long bits64(const double* p) { return __double_as_longlong(__ldg(p)); }
+template <class R> __device__ __forceinline__ bool step_finite(R v) { return isfinite(v); }
+template <> __device__ __forceinline__ bool step_finite<double>(double v) { return finite64(v); }
+
+// largest i in [0, n-1] with s >= face_i ---------------------------------------
+__device__ __forceinline__ int cell_uniform(double s, float inv_h, int n, const double* f) {
+    int i = (int)(lead_f32(s) * inv_h);
     i = min(max(i, 0), n - 1);
-    while (i > 0 && s < (double)i * h) --i;
-    while (i < n - 1 && s >= (double)(i + 1) * h) ++i;
+    const long long b = order64(s);
+    while (i > 0 && b < bits64(f + i)) --i;
+    while (i < n - 1 && b >= bits64(f + i + 1)) ++i;
     return i;
 }
 __device__ __forceinline__ int cell_uniform(float s, float inv_h, int n, const float* f_up) {
@@ -99,13 +122,15 @@ __device__ __forceinline__ int cell_uniform(float s, float inv_h, int n, const f
 }
 template <class R>
 __device__ __forceinline__ int cell_y(R y, const StepArgs<R>& a) {
-    int b = (int)(y * a.ybin_scale);
+    int b;
+    if constexpr (sizeof(R) == 8) b = (int)(lead_f32(y) * a.ybin_scalef);
+    else b = (int)(y * a.ybin_scale);
     b = min(max(b, 0), a.ybins - 1);
     int j = a.ybin[b];
-    if (sizeof(R) == 8) {
-        const double yd = (double)y;
-        while (j > 0 && yd < a.yf[j]) --j;
-        while (j < a.ny - 1 && yd >= a.yf[j + 1]) ++j;
+    if constexpr (sizeof(R) == 8) {
+        const long long yb = order64(y);
+        while (j > 0 && yb < bits64(a.yf + j)) --j;
+        while (j < a.ny - 1 && yb >= bits64(a.yf + j + 1)) ++j;
     } else {
         const float yfl = (float)y;
         while (j > 0 && yfl < a.yf_up[j]) --j;
@@ -135,8 +160,8 @@ template <class R>
 __device__ __forceinline__ uint32_t cell_key(R x, R y, R z, const StepArgs<R>& a, int* jout) {
     int i, k;
     if constexpr (sizeof(R) == 8) {
-        i = cell_uniform((double)x, a.dx, a.nx, a.xf_up, 0.0);
-        k = cell_uniform((double)z, a.dz, a.nz, a.zf_up, 0.0);
+        i = cell_uniform((double)x, a.inv_dxf, a.nx, a.xf);
+        k = cell_uniform((double)z, a.inv_dzf, a.nz, a.zf);
     } else {
         i = cell_uniform((float)x, (float)a.inv_dx, a.nx, a.xf_up);
         k = cell_uniform((float)z, (float)a.inv_dz, a.nz, a.zf_up);
@@ -154,15 +179,17 @@ __device__ __forceinline__ uint32_t cell_key_near(R x, R y, R z, const StepArgs<
                                                   const YRow* rg = nullptr) {
     int i, k;
     if constexpr (sizeof(R) == 8) {
-        i = cell_uniform((double)x, a.dx, a.nx, a.xf_up, 0.0);
-        k = cell_uniform((double)z, a.dz, a.nz, a.zf_up, 0.0);
+        i = cell_uniform((double)x, a.inv_dxf, a.nx, a.xf);
+        k = cell_uniform((double)z, a.inv_dzf, a.nz, a.zf);
     } else {
         i = cell_uniform((float)x, (float)a.inv_dx, a.nx, a.xf_up);
         k = cell_uniform((float)z, (float)a.inv_dz, a.nz, a.zf_up);
     }
     bool in;
-    if constexpr (sizeof(R) == 8) in = (double)y >= a.yf[jg] && (double)y < a.yf[jg + 1];
-    else if (rg) in = (float)y >= rg->f.x && (float)y < rg->f.y;
+    if constexpr (sizeof(R) == 8) {
+        const long long yb = order64(y);
+        in = yb >= bits64(a.yf + jg) && yb < bits64(a.yf + jg + 1);
+    } else if (rg) in = (float)y >= rg->f.x && (float)y < rg->f.y;
     else in = (float)y >= a.yf_up[jg] && (float)y < a.yf_up[jg + 1];
     const int j = in ? jg : cell_y(y, a);
     *jout = j;
@@ -184,16 +211,34 @@ template <class R>
 __device__ __forceinline__ void corners(const StepArgs<R>& a, R x, R y, R z, int j, Corners<R>& cr,
                                         unsigned int* err, const YRow* yr = nullptr) {
     R sx = x * a.inv_dx - (R)0.5;
-    R fx = rfloor(sx);
-    R wx = sx - fx;
     R sz = z * a.inv_dz - (R)0.5;
-    R fz = rfloor(sz);
-    R wz = sz - fz;
-    if (!(fx >= (R)-1 && fx <= (R)(a.nx - 1)) || !(fz >= (R)-1 && fz <= (R)(a.nz - 1))) {
-        *err |= TRIBO_DEV_OUTSIDE;
-        fx = 0; fz = 0; wx = 0; wz = 0;
+    R wx, wz;
+    int i0, k0;
+    if constexpr (sizeof(R) == 8) {
+        // floor by one addition rounded down: below 2^31 the sum's low word is the integer
+        const double big = 6755399441055744.0;                 // 1.5 * 2^52
+        const double tx = __dadd_rd(sx, big), tz = __dadd_rd(sz, big);
+        i0 = __double2loint(tx);
+        k0 = __double2loint(tz);
+        wx = sx - (tx - big);
+        wz = sz - (tz - big);
+        const bool in = (__double2hiint(sx) & 0x7fffffff) < 0x41e00000 && (__double2hiint(sz) & 0x7fffffff) < 0x41e00000;
+        if (!in || i0 < -1 || i0 > a.nx - 1 || k0 < -1 || k0 > a.nz - 1) {
+            *err |= TRIBO_DEV_OUTSIDE;
+            i0 = 0; k0 = 0; wx = 0; wz = 0;
+        }
+    } else {
+        R fx = rfloor(sx);
+        wx = sx - fx;
+        R fz = rfloor(sz);
+        wz = sz - fz;
+        if (!(fx >= (R)-1 && fx <= (R)(a.nx - 1)) || !(fz >= (R)-1 && fz <= (R)(a.nz - 1))) {
+            *err |= TRIBO_DEV_OUTSIDE;
+            fx = 0; fz = 0; wx = 0; wz = 0;
+        }
+        i0 = (int)fx;
+        k0 = (int)fz;
     }
-    int i0 = (int)fx, k0 = (int)fz;
     int i1 = i0 + 1, k1 = k0 + 1;
     if (i0 < 0) i0 += a.nx;
     if (i1 >= a.nx) i1 -= a.nx;
@@ -207,7 +252,8 @@ __device__ __forceinline__ void corners(const StepArgs<R>& a, R x, R y, R z, int
         cr.inv_dy = (R)(up ? yr->g.y : yr->g.x);
         wy = (y - (R)(up ? yr->f.w : yr->f.z)) * cr.inv_dy;
     } else {
-        jn0 = (y >= a.Yr[j + 1]) ? j + 1 : j;
+        if constexpr (sizeof(R) == 8) jn0 = order64(y) >= bits64(a.Yr + j + 1) ? j + 1 : j;
+        else jn0 = (y >= a.Yr[j + 1]) ? j + 1 : j;
         cr.inv_dy = a.invdY[jn0];
         wy = (y - a.Yr[jn0]) * cr.inv_dy;
     }
@@ -282,6 +328,31 @@ __device__ __forceinline__ R phi2_of(R s, R phi1) {
         return s * s * p;
     }
     return s - phi1;
+}
+
+// phi1 = 1 - e^-s and phi2 = s - phi1 in FP64: below 1/2 both come from the one series, phi1 = s - s^2 p (s^2 p < s / 4, so the difference
+// rounds once), in place of an expm1; a step is a small fraction of tau, and below 1/64 seven
+// terms leave the truncation below the epsilon (the eighth is s^7 2 / 9! < 2^-59 of p)
+__device__ __forceinline__ void phi12(double s, double& phi1, double& phi2) {
+    if (s < 0.5) {
+        constexpr Phi2Series<16> S{};
+        double p;
+        if (s < 0.015625) {
+            p = S.c[6];
+#pragma unroll
+            for (int k = 5; k >= 0; --k) p = S.c[k] + s * p;
+        } else {
+            p = S.c[16];
+#pragma unroll
+            for (int k = 15; k >= 0; --k) p = S.c[k] + s * p;
+        }
+        const double sp = s * p;
+        phi1 = s - s * sp;
+        phi2 = s * sp;
+    } else {
+        phi1 = -rexpm1(-s);
+        phi2 = s - phi1;
+    }
 }
 
 // the condenser-model charge of one wall impact (FP64)
@@ -366,7 +437,9 @@ StepArgs<R> make_args(tribo_ctx* c, double dt) {
     a.inv_dx = (R)(1.0 / c->dx); a.inv_dz = (R)(1.0 / c->dz);
     a.inv_lx = (R)(1.0 / c->lx); a.inv_lz = (R)(1.0 / c->lz);
     a.dt = (R)dt;
-    a.dx = c->dx; a.dz = c->dz;
+    a.xf = c->d_xf; a.zf = c->d_zf;
+    a.inv_dxf = (float)(1.0 / c->dx); a.inv_dzf = (float)(1.0 / c->dz);
+    a.ybin_scalef = (float)((double)c->ybins / c->ly);
     a.yf = c->d_yf; a.yf_up = c->d_yf_up; a.xf_up = c->d_xf_up; a.zf_up = c->d_zf_up;
     a.ybin = c->d_ybin; a.ybins = c->ybins; a.ybin_scale = (R)((double)c->ybins / c->ly);
     a.Yr = (const R*)c->d_Yr; a.invdY = (const R*)c->d_invdY;
@@ -466,8 +539,13 @@ __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, i
             else tau = tau_p / ((R)1 + rpow23(re) / (R)6);
         }
         const R s = a.dt / tau;
-        const R phi1 = -rexpm1(-s);
-        const R phi2 = phi2_of(s, phi1);
+        R phi1, phi2;
+        if constexpr (sizeof(R) == 8) {
+            phi12(s, phi1, phi2);
+        } else {
+            phi1 = -rexpm1(-s);
+            phi2 = phi2_of(s, phi1);
+        }
         const R tx = uf[0] + ax * tau, ty = uf[1] + ay * tau, tz = uf[2] + az * tau;
         vxn = vx + (tx - vx) * phi1;
         vyn = vy + (ty - vy) * phi1;
@@ -487,13 +565,17 @@ __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, i
             atomicAdd(&a.fs[2 * a.ncell + key0], w * ((uf[2] - vz) * phi1 - az * tp));
         }
     }
-    // periodic wrap in x and z (FP64: the oracle's own operations, so cells stay bit-exact;
-    // FP32: the reciprocal, with both ends corrected)
+    // periodic wrap in x and z (FP64: the oracle's own operations, so cells stay bit-exact; inside
+    // [0, l) they change nothing and are passed by; FP32: the reciprocal, with both ends corrected)
     if constexpr (sizeof(R) == 8) {
-        xn = xn - a.lx * rfloor(xn / a.lx);
-        if (xn >= a.lx) xn -= a.lx;
-        zn = zn - a.lz * rfloor(zn / a.lz);
-        if (zn >= a.lz) zn -= a.lz;
+        if ((unsigned long long)__double_as_longlong(xn) >= (unsigned long long)__double_as_longlong(a.lx)) {
+            xn = xn - a.lx * rfloor(xn / a.lx);
+            if (xn >= a.lx) xn -= a.lx;
+        }
+        if ((unsigned long long)__double_as_longlong(zn) >= (unsigned long long)__double_as_longlong(a.lz)) {
+            zn = zn - a.lz * rfloor(zn / a.lz);
+            if (zn >= a.lz) zn -= a.lz;
+        }
     } else {
         xn = xn - a.lx * rfloor(xn * a.inv_lx);
         if (xn < (R)0) xn += a.lx;
@@ -535,7 +617,7 @@ __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, i
         atomicAdd(&a.acc->sum_wall, dq);
         atomicAdd(&a.acc->n_impacts, 1ull);
     }
-    if (!(rfinite(xn) && rfinite(yn) && rfinite(zn) && rfinite(vxn) && rfinite(vyn) && rfinite(vzn)))
+    if (!(step_finite(xn) && step_finite(yn) && step_finite(zn) && step_finite(vxn) && step_finite(vyn) && step_finite(vzn)))
         err |= TRIBO_DEV_NONFINITE;
     X[n] = xn; Y[n] = yn; Z[n] = zn;
     VX[n] = vxn; VY[n] = vyn; VZ[n] = vzn;

@@ -33,8 +33,12 @@ namespace tribo {
 
 namespace {
 
+// FP64: bound by the FP64 pipe (two lanes a SM and clock): about 135 operations a particle, of which
+// the gather is 60 and the two divisions 18, 0.23 ms of the pipe for 1M particles.  Measured 295 us
+// (481 before the locate, the compares, the wrap and expm1 left the FP64 pipe); 80 registers, three
+// blocks a SM, hold it without spilling.  FP32: see the loop.
 template <class R>
-__global__ void __launch_bounds__(kStepThreads, kStepMinBlocks) k_step(StepArgs<R> a, PView p, int write_cell) {
+__global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(StepArgs<R> a, PView p, int write_cell) {
     pdl_wait();
     extern __shared__ unsigned int sh_hist[];
     const bool use_hist = a.hist != nullptr;
@@ -112,10 +116,13 @@ tribo_status step_impl(tribo_ctx* c, const PView& p, double dt, bool deposit_nex
     a.fs_coef = (R)io.fs_coef;
     const size_t sh = sizeof(unsigned int) * (size_t)c->ny;
     phase_begin(c, PH_STEP);
-    // one resident wave (a grid of several waves measured 6% slower)
-    const int kblocks = (int)std::min<int64_t>((p.n + kStepThreads - 1) / kStepThreads,
-                                               (int64_t)c->num_sms * kStepMinBlocks);
-    (void)launch_pdl(k_step<R>, dim3(kblocks), dim3(kStepThreads), sh, c->stream, a, p, write_cell ? 1 : 0);
+    // one resident wave (a grid of several waves measured 6% slower); a few particles in small
+    // blocks, so that they spread over the SMs (in FP64 a block of 256 keeps one SM's two FP64 lanes
+    // busy for its whole step: 2000 particles 23.3 -> 13.4 us)
+    const int threads = p.n <= (int64_t)c->num_sms * kStepThreads ? 64 : kStepThreads;
+    const int kblocks = (int)std::min<int64_t>((p.n + threads - 1) / threads,
+                                               (int64_t)c->num_sms * step_min_blocks<R>() * (kStepThreads / threads));
+    (void)launch_pdl(k_step<R>, dim3(kblocks), dim3(threads), sh, c->stream, a, p, write_cell ? 1 : 0);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }

@@ -133,6 +133,10 @@ tribo_status build_tables(tribo_ctx* c) {
     TRIBO_CUDA(cudaMalloc(&c->d_invdY, rs * (ny + 1)));
     TRIBO_CUDA(cudaMalloc(&c->d_inv_vol, rs * ny));
     if (c->prec == TRIBO_FP64) {
+        std::vector<double> xd(nx + 1), zd(nz + 1);
+        for (int i = 0; i <= nx; ++i) xd[i] = (double)i * c->dx;
+        for (int k = 0; k <= nz; ++k) zd[k] = (double)k * c->dz;
+        if ((st = upload(&c->d_xf, xd)) || (st = upload(&c->d_zf, zd))) return st;
         TRIBO_CUDA(cudaMemcpy(c->d_Yr, Yd.data(), rs * (ny + 2), cudaMemcpyHostToDevice));
         TRIBO_CUDA(cudaMemcpy(c->d_invdY, inv.data(), rs * (ny + 1), cudaMemcpyHostToDevice));
         TRIBO_CUDA(cudaMemcpy(c->d_inv_vol, ivol.data(), rs * ny, cudaMemcpyHostToDevice));
@@ -396,7 +400,7 @@ void free_ctx(tribo_ctx* c) {
     poisson_free(c);
     modes_free(c);
     void* ptrs[] = {c->d_yf, c->d_Y, c->d_scale_q, c->d_scale_rho, c->d_yf_up, c->d_xf_up, c->d_zf_up,
-                    c->d_ybin, c->d_Yr, c->d_invdY, c->d_yrow, c->u_lat, c->E_lat, c->Q, c->stage, c->d_acc,
+                    c->d_xf, c->d_zf, c->d_ybin, c->d_Yr, c->d_invdY, c->d_yrow, c->u_lat, c->E_lat, c->Q, c->stage, c->d_acc,
                     c->d_hist, c->d_scalar, c->alt, c->sort_counts, c->sort_key, c->sort_rank, c->sort_perm,
                     c->sort_tiles, c->adj, c->nf_members, c->nf_acc, c->pp_partner, c->d_inv_vol,
                     c->adj_E, c->n_imp0, c->patch};

@@ -94,6 +94,8 @@ struct tribo_ctx {
     double* d_Y = nullptr;       // ny+2 lattice nodes
     double* d_scale_q = nullptr; // ny: -1 / (eps V_j) (charge sum -> RHS)
     double* d_scale_rho = nullptr; // ny: -1 / eps (density -> RHS)
+    double* d_xf = nullptr;      // nx+1, nz+1 FP64 faces i dx, k dz (FP64 mode)
+    double* d_zf = nullptr;
     float* d_yf_up = nullptr;    // ny+1: smallest float >= yf
     float* d_xf_up = nullptr;    // nx+1
     float* d_zf_up = nullptr;    // nz+1
