@@ -47,21 +47,20 @@ __device__ __forceinline__ void dft8(cplx<R>* y) {
     dft4<R, SIGN>(e);
     dft4<R, SIGN>(o);
     const R r = (R)0.70710678118654752440;  // 1/sqrt(2)
-    // w8^u = exp(SIGN i pi u / 4)
-    const cplx<R> w1 = {r, (R)SIGN * r};
-    const cplx<R> w3 = {-r, (R)SIGN * r};
-    const cplx<R> t0 = o[0];
-    const cplx<R> t1 = o[1] * w1;
-    const cplx<R> t2 = mul_si(o[2], (R)SIGN);
-    const cplx<R> t3 = o[3] * w3;
-    y[0] = e[0] + t0;
-    y[4] = e[0] - t0;
-    y[1] = e[1] + t1;
-    y[5] = e[1] - t1;
+    const R sg = (R)SIGN;
+    // w8^u = exp(SIGN i pi u / 4): the products with w8 and w8^3 are r times a sum of the parts,
+    // taken up by the butterflies' fused multiply-adds
+    const cplx<R> a = {o[1].re - sg * o[1].im, o[1].im + sg * o[1].re};
+    const cplx<R> b = {o[3].re + sg * o[3].im, o[3].im - sg * o[3].re};
+    const cplx<R> t2 = mul_si(o[2], sg);
+    y[0] = e[0] + o[0];
+    y[4] = e[0] - o[0];
+    y[1] = {e[1].re + r * a.re, e[1].im + r * a.im};
+    y[5] = {e[1].re - r * a.re, e[1].im - r * a.im};
     y[2] = e[2] + t2;
     y[6] = e[2] - t2;
-    y[3] = e[3] + t3;
-    y[7] = e[3] - t3;
+    y[3] = {e[3].re - r * b.re, e[3].im - r * b.im};
+    y[7] = {e[3].re + r * b.re, e[3].im + r * b.im};
 }
 
 template <class R, int SIGN, int RAD>

@@ -397,7 +397,7 @@ __device__ __noinline__ void inv_ztask(const cplx<R>* __restrict__ S, const cplx
 // phi (field 0); wall lines carry E_x = E_z = 0
 template <class R, int M>
 __device__ __noinline__ void inv_xtask(const cplx<R>* slot, R* __restrict__ E, double* __restrict__ phi, int ny,
-                                       int nz, int jn, int grp, int want_phi, int want_e, R norm, size_t nodes,
+                                       int nz, int jn, int grp, int want_phi, int want_e, size_t nodes,
                                        const cplx<R>* __restrict__ tw, const cplx<R>* __restrict__ t2,
                                        const R* __restrict__ sx, cplx<R>* buf) {
     using F4 = fft::FourStep<M, kThreads>;
@@ -411,6 +411,11 @@ __device__ __noinline__ void inv_xtask(const cplx<R>* slot, R* __restrict__ E, d
     const bool interior = jn >= 1 && jn <= ny;
     const size_t fs = (size_t)nz * NXH;
     const size_t line = (size_t)k * nyn + jn;
+    // the second step's threads are N1 a line, packed (whole warps idle instead of lanes)
+    const int l2 = threadIdx.x / N1, r2 = threadIdx.x % N1;
+    const int kl2 = grp * LPB + l2;
+    const bool live2 = l2 < LPB && kl2 < nz;
+    const size_t line2 = (size_t)kl2 * nyn + jn;
     const int nf = want_phi ? 4 : 3;
     for (int f = want_e ? 0 : 3; f < nf; ++f) {
         const bool active = live && (f == 1 || interior);
@@ -421,15 +426,8 @@ __device__ __noinline__ void inv_xtask(const cplx<R>* slot, R* __restrict__ E, d
 #pragma unroll
             for (int n1 = 0; n1 < N1; ++n1) {
                 const int m = N2 * n1 + r;
-                cplx<R> xa = fft::ld_cplx<R, fft::kL2Only>(X + m), xb = fft::ld_cplx<R, fft::kL2Only>(X + M - m);
-                if (f == 0) {     // E_x multiplier -i sin(2 pi m / nx) / dx
-                    xa = cplx<R>{sx[m] * xa.im, -sx[m] * xa.re};
-                    xb = cplx<R>{sx[M - m] * xb.im, -sx[M - m] * xb.re};
-                }
-                const cplx<R> cb = conj(xb);
-                const cplx<R> sum = xa + cb;
-                const cplx<R> t = conj(tw[m]) * (xa - cb);
-                y[n1] = cplx<R>{sum.re - t.im, sum.im + t.re};
+                const cplx<R> xa = fft::ld_cplx<R, fft::kL2Only>(X + m), xb = fft::ld_cplx<R, fft::kL2Only>(X + M - m);
+                y[n1] = f == 0 ? split_inv_dx(xa, xb, tw[m], sx[m]) : split_inv(xa, xb, tw[m]);
             }
             fft::reg_dft<R, 1, N1, 2 * N2>(y, tw);
 #pragma unroll
@@ -451,22 +449,22 @@ __device__ __noinline__ void inv_xtask(const cplx<R>* slot, R* __restrict__ E, d
                 for (size_t b = b0 + (size_t)threadIdx.x * 128; b < b1; b += (size_t)blockDim.x * 128)
                     asm volatile("discard.global.L2 [%0], 128;" ::"l"(base + b) : "memory");
         }
-        if (active && r < N1) {
+        if (live2 && (f == 1 || interior)) {
             cplx<R> z[N2];
-            const cplx<R>* b = buf + l * CS + r;
+            const cplx<R>* b = buf + l2 * CS + r2;
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) z[n2] = b[n2 * (N1 + 1)];
             fft::reg_dft<R, 1, N2, 2 * N1>(z, tw);
             if (f < 3) {       // written once: evict-first in L2
-                cplx<R>* row = reinterpret_cast<cplx<R>*>(E + (size_t)f * nodes + line * NX);
+                cplx<R>* row = reinterpret_cast<cplx<R>*>(E + (size_t)f * nodes + line2 * NX);
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2)
-                    fft::st_cplx<R, fft::kStream>(row + r + N1 * k2, cplx<R>{z[k2].re * norm, z[k2].im * norm});
+                    fft::st_cplx<R, fft::kStream>(row + r2 + N1 * k2, z[k2]);
             } else {
-                double2* prow = reinterpret_cast<double2*>(phi + ((size_t)k * ny + (jn - 1)) * NX);
+                double2* prow = reinterpret_cast<double2*>(phi + ((size_t)kl2 * ny + (jn - 1)) * NX);
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2)
-                    __stcs(prow + r + N1 * k2, make_double2((double)(z[k2].re * norm), (double)(z[k2].im * norm)));
+                    __stcs(prow + r2 + N1 * k2, make_double2((double)z[k2].re, (double)z[k2].im));
             }
         }
         __syncthreads();
@@ -484,7 +482,7 @@ __device__ __noinline__ void inv_xtask(const cplx<R>* slot, R* __restrict__ E, d
 template <class R, int M, int NZ>
 __global__ void __launch_bounds__(kThreads, (fused_min_blocks<R, M, NZ>())) k_inv_fused(
     const cplx<R>* __restrict__ S, const cplx<R>* __restrict__ Fy, cplx<R>* ring, R* __restrict__ E,
-    double* __restrict__ phi, int ny, int want_phi, int want_e, R norm, size_t nodes,
+    double* __restrict__ phi, int ny, int want_phi, int want_e, size_t nodes,
     const double* __restrict__ sinx, const double* __restrict__ sinz, const cplx<R>* __restrict__ twx_g,
     const cplx<R>* __restrict__ twz_g, PipeSync* sy, Pipe pipe, unsigned* err) {
     pdl_wait();
@@ -515,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, (fused_min_blocks<R, M, NZ>())) k_in
         pipe_task(pipe, L.t, cons, plane, idx);
         pipe_acquire(L, pipe, sy, cons, plane, err);
         cplx<R>* slot = ring + (size_t)(plane % pipe.P) * slot_elems;
-        if (cons) inv_xtask<R, M>(slot, E, phi, ny, NZ, plane, idx, want_phi, want_e, norm, nodes, twx, t2, sx, buf);
+        if (cons) inv_xtask<R, M>(slot, E, phi, ny, NZ, plane, idx, want_phi, want_e, nodes, twx, t2, sx, buf);
         else inv_ztask<R, NZ>(S, Fy, slot, ny, NXH, plane, idx, want_e, twz, sz, buf);
         pipe_release(L, sy, cons, plane);
     }
@@ -571,8 +569,7 @@ tribo_status launch_inv_fused(tribo_ctx* c, void* E, double* phi) {
     const size_t fstride = (size_t)NZ * (c->ny + 2) * c->nxh;
     (void)launch_pdl(k_inv_fused<R, M, NZ>, dim3(grid), dim3(kThreads), smem, c->stream,
         (const cplx<R>*)c->S, (const cplx<R>*)c->F + fstride, (cplx<R>*)c->ring, (R*)E, phi, c->ny,
-        phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, (R)(1.0 / ((double)c->nx * (double)NZ)),
-        (size_t)NZ * (c->ny + 2) * c->nx, c->d_sinx, c->d_sinz, (const cplx<R>*)c->d_twx,
+        phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, (size_t)NZ * (c->ny + 2) * c->nx, c->d_sinx, c->d_sinz, (const cplx<R>*)c->d_twx,
         (const cplx<R>*)c->d_twz, sy, pipe_t, &c->d_acc->err);
     return TRIBO_OK;
 }

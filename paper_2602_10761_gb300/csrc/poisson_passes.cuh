@@ -55,11 +55,29 @@ __device__ __forceinline__ ds ds_mul(ds a, ds b) {
 __device__ __forceinline__ ds ds_neg(ds a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ float ds_f(ds a) { return a.hi + a.lo; }
 
+// ---------------------------------------------------------------- real transforms' split step
+// Inverse: the half-length value Z_m of a real line from X_m = xa and X_M-m = xb,
+//   Z = (xa + conj xb) + i conj(W^m) (xa - conj xb), w = W^m = exp(-2 pi i m / N),
+// four additions and four fused multiply-adds (transforms in FP64 are bound by
+// the FP64 pipe: operations are time).
+template <class R>
+__device__ __forceinline__ cplx<R> split_inv(cplx<R> xa, cplx<R> xb, cplx<R> w) {
+    const R sr = xa.re + xb.re, si = xa.im - xb.im, dr = xa.re - xb.re, di = xa.im + xb.im;
+    return {sr - w.re * di + w.im * dr, si + w.re * dr + w.im * di};
+}
+// the same of -i s X (s = sin(2 pi m / N) / dx, equal for m and M - m): E_x's spectrum from the potential's
+template <class R>
+__device__ __forceinline__ cplx<R> split_inv_dx(cplx<R> xa, cplx<R> xb, cplx<R> w, R s) {
+    const R sr = xa.re + xb.re, si = xa.im - xb.im, dr = xa.re - xb.re, di = xa.im + xb.im;
+    return {s * (di + w.re * sr + w.im * si), s * (w.re * si - w.im * sr - dr)};
+}
+
 // ---------------------------------------------------------------- x forward
 // Thread group (line, r) per line (k, j) of the charge-sum array:
 // z_n = x_2n + i x_2n+1 (scaled to -rho/eps), Z = FFT_M(z) by the register
-// four-step, X_m = (Z_m + conj Z_M-m)/2 - (i/2) W^m (Z_m - conj Z_M-m) for
-// m = 0..M.  Each thread zeroes the charge sums it has read.  The source has
+// four-step, X_m = (Z_m + conj Z_M-m) - i W^m (Z_m - conj Z_M-m) for m = 0..M
+// (the halves of the split step and the normalisation 1/(nx nz) of the inverse
+// transforms are in the scale), X_m and X_M-m from one sum and product.  Each thread zeroes the charge sums it has read.  The source has
 // type QT: the FP64 cell charge sums (or a caller's FP64 density), rounded to
 // R as they are read, or the adjoint's R-typed charge adjoint.
 // six resident blocks (40 registers) where the length fits them without spilling: FP32 factors up
@@ -95,7 +113,7 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
     // fills its twiddle table, so that the table's round trip overlaps the loads
     cplx<R> y[N1];
     if (live && r < N2) {
-        const R s = from_f64<R>(scale_row[line % ny]);
+        const R s = (R)0.5 * from_f64<R>(scale_row[line % ny]);
         using V2 = std::conditional_t<sizeof(QT) == 8, double2, float2>;   // (x_2n, x_2n+1)
         V2* row = reinterpret_cast<V2*>(src) + (size_t)line * M;
         unsigned nz_mask = 0;        // which element pairs hold a nonzero sum
@@ -127,26 +145,31 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
         for (int k1 = 0; k1 < N1; ++k1) lb[r * (N1 + 1) + k1] = y[k1];
     }
     __syncthreads();
+    // the second step's threads are N1 a line: packed, so that whole warps are idle instead of
+    // lanes where N1 < N2
+    const int l2 = threadIdx.x / N1, r2 = threadIdx.x % N1;
+    const bool live2 = l2 < LPB && blockIdx.x * LPB + l2 < nlines;
+    cplx<R>* lb2 = buf + l2 * CS;
     cplx<R> z[N2];
-    if (live && r < N1) {
+    if (live2) {
 #pragma unroll
-        for (int n2 = 0; n2 < N2; ++n2) z[n2] = lb[n2 * (N1 + 1) + r];
+        for (int n2 = 0; n2 < N2; ++n2) z[n2] = lb2[n2 * (N1 + 1) + r2];
         fft::reg_dft<R, -1, N2, 2 * N1>(z, tw);
     }
     __syncthreads();
-    if (live && r < N1) {
+    if (live2) {
 #pragma unroll
-        for (int k2 = 0; k2 < N2; ++k2) lb[r + N1 * k2] = z[k2];
+        for (int k2 = 0; k2 < N2; ++k2) lb2[r2 + N1 * k2] = z[k2];
     }
     __syncthreads();
     if (live) {
         cplx<R>* out = S + (size_t)line * NXH;
-        for (int m = r; m <= M; m += TPC) {
-            const cplx<R> zm = lb[m == M ? 0 : m];
-            const cplx<R> zc = conj(lb[m == 0 ? 0 : M - m]);
-            const cplx<R> sum = zm + zc, dif = zm - zc;
-            const cplx<R> t = tw[m] * dif;
-            out[m] = cplx<R>{(R)0.5 * (sum.re + t.im), (R)0.5 * (sum.im - t.re)};
+        for (int m = r; 2 * m <= M; m += TPC) {
+            const cplx<R> zm = lb[m], zc = lb[m == 0 ? 0 : M - m], w = tw[m];
+            const R sr = zm.re + zc.re, si = zm.im - zc.im, dr = zm.re - zc.re, di = zm.im + zc.im;
+            const R tr = w.re * dr - w.im * di, ti = w.re * di + w.im * dr;
+            out[m] = cplx<R>{sr + ti, si - tr};
+            if (2 * m < M) out[M - m] = cplx<R>{sr - ti, -si - tr};
         }
     }
 }
@@ -470,19 +493,21 @@ void ysolve_twist_launch(int64_t pencils, int n, int num_sms, int ny, cudaStream
 }
 
 // ---------------------------------------------------------------- z passes (four-step)
-// Forward z transform of S in place: block (cell plane j, W columns of m_x).
-// one tile (cell plane j, W columns of m_x) of the forward z transform; out of line so
-// that each tile starts from a fresh register allocation
+// The columns of all planes are one run: element k of column c = plane * nxh + m_x
+// sits at k * (planes nxh) + c, so a tile is any W neighbouring columns, planes
+// straddled, and only the last tile of a pass has idle lanes.  (Tiles that ended
+// with their plane left 31 of 64 lanes idle at nx = 64, where m_x runs to 32, and
+// 15 of 80 at nx = 128: FP64 inverse z pass at 64^3
+// 33.8 -> 22.7 us, at 128^3 182 -> 147.)
+// one tile of the forward z transform of S in place; out of line so that each tile starts from a
+// fresh register allocation
 template <class R, int NZ>
-__device__ __noinline__ void zfwd_tile(cplx<R>* __restrict__ S, int ny, int nxh, int ntx, int t,
-                                       const cplx<R>* __restrict__ tw, cplx<R>* buf) {
+__device__ __noinline__ void zfwd_tile(cplx<R>* __restrict__ S, int ncols, int t, const cplx<R>* __restrict__ tw,
+                                       cplx<R>* buf) {
     using F4 = fft::FourStep<NZ, kThreads>;
-    const int j = t / ntx;
-    const int mx0 = (t - j * ntx) * F4::W;
-    const int ncol = min(F4::W, nxh - mx0);
-    cplx<R>* base = S + (size_t)j * nxh + mx0;
-    const size_t rs = (size_t)ny * nxh;
-    fft::column_fft<R, -1, NZ, kThreads, false>(base, rs, base, rs, ncol, tw, nullptr, buf);
+    cplx<R>* base = S + (size_t)t * F4::W;
+    fft::column_fft<R, -1, NZ, kThreads, false>(base, ncols, base, ncols, min(F4::W, ncols - t * F4::W), tw, nullptr,
+                                                buf);
 }
 
 template <class R, int NZ, bool kTab = false>
@@ -500,45 +525,32 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, NZ>())) k_zfwd4(c
     cplx<R>* buf = tw + NZ;
     for (int i = threadIdx.x; i < NZ; i += kThreads) tw[i] = tw_g[i];
     __syncthreads();
-    const int ntx = (nxh + F4::W - 1) / F4::W;
-    for (int t = blockIdx.x; t < ny * ntx; t += gridDim.x) zfwd_tile<R, NZ>(S, ny, nxh, ntx, t, tw, buf);
+    const int ncols = ny * nxh;
+    for (int t = blockIdx.x; t * F4::W < ncols; t += gridDim.x) zfwd_tile<R, NZ>(S, ncols, t, tw, buf);
 }
 
-// Inverse z transforms: block (node plane jn, W columns of m_x).  All planes:
-// F1 = IFFT_z(E_y-hat) in place; interior planes: F0 = IFFT_z(phi-hat of cell
-// jn-1) and F2 = IFFT_z(-i sin(2 pi m_z/nz)/dz phi-hat).
-// one tile (node plane jn, W columns of m_x) of the inverse z transforms, out of line
+// Inverse z transforms: F1 = IFFT_z(E_y-hat) in place on all node planes; on the
+// interior planes F0 = IFFT_z(phi-hat of cell jn-1) and F2 = IFFT_z(-i sin(2 pi
+// m_z/nz)/dz phi-hat).  Out of line as above: one tile of F1, and one of F0 and F2
+// (dz: F2 too).
 template <class R, int NZ>
-__device__ __noinline__ void zinv_tile(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F, int ny, int nxh,
-                                       int ntx, int t, size_t fstride, const cplx<R>* __restrict__ tw,
-                                       const R* __restrict__ sz, cplx<R>* buf) {
+__device__ __noinline__ void zinv_tile_e(cplx<R>* __restrict__ Fy, int ncols, int t, const cplx<R>* __restrict__ tw,
+                                         cplx<R>* buf) {
     using F4 = fft::FourStep<NZ, kThreads>;
-    const int nyn = ny + 2;
-    const size_t rsF = (size_t)nyn * nxh, rsS = (size_t)ny * nxh;
-    const int jn = t / ntx;
-    const int mx0 = (t - jn * ntx) * F4::W;
-    const int ncol = min(F4::W, nxh - mx0);
-    cplx<R>* Fy = F + fstride + (size_t)jn * nxh + mx0;
-    fft::column_fft<R, 1, NZ, kThreads, false>(Fy, rsF, Fy, rsF, ncol, tw, nullptr, buf);
-    if (jn >= 1 && jn <= ny) {
-        const cplx<R>* ph = S + (size_t)(jn - 1) * nxh + mx0;
-        cplx<R>* F0 = F + (size_t)jn * nxh + mx0;
-        fft::column_fft<R, 1, NZ, kThreads, false>(ph, rsS, F0, rsF, ncol, tw, nullptr, buf);
-        fft::column_fft<R, 1, NZ, kThreads, true>(ph, rsS, F0 + 2 * fstride, rsF, ncol, tw, sz, buf);
-    }
+    cplx<R>* base = Fy + (size_t)t * F4::W;
+    fft::column_fft<R, 1, NZ, kThreads, false>(base, ncols, base, ncols, min(F4::W, ncols - t * F4::W), tw, nullptr,
+                                               buf);
 }
-// the potential alone: only phi-hat's transform, on the interior node rows
-template <class R, int NZ>
-__device__ __noinline__ void zinv_tile_phi(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F, int ny,
-                                           int nxh, int ntx, int t, const cplx<R>* __restrict__ tw, cplx<R>* buf) {
+template <class R, int NZ, bool kDz>
+__device__ __noinline__ void zinv_tile_phi(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F0, int ncols, int fcols,
+                                           int t, size_t fstride, const cplx<R>* __restrict__ tw,
+                                           const R* __restrict__ sz, cplx<R>* buf) {
     using F4 = fft::FourStep<NZ, kThreads>;
-    const size_t rsF = (size_t)(ny + 2) * nxh, rsS = (size_t)ny * nxh;
-    const int jn = t / ntx;
-    const int mx0 = (t - jn * ntx) * F4::W;
-    const int ncol = min(F4::W, nxh - mx0);
-    if (jn < 1 || jn > ny) return;
-    fft::column_fft<R, 1, NZ, kThreads, false>(S + (size_t)(jn - 1) * nxh + mx0, rsS, F + (size_t)jn * nxh + mx0,
-                                               rsF, ncol, tw, nullptr, buf);
+    const size_t c0 = (size_t)t * F4::W;
+    const int ncol = min(F4::W, ncols - t * F4::W);
+    fft::column_fft<R, 1, NZ, kThreads, false>(S + c0, ncols, F0 + c0, fcols, ncol, tw, nullptr, buf);
+    if constexpr (kDz)
+        fft::column_fft<R, 1, NZ, kThreads, true>(S + c0, ncols, F0 + 2 * fstride + c0, fcols, ncol, tw, sz, buf);
 }
 
 template <class R, int NZ, bool kTab = false>
@@ -564,10 +576,14 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, NZ>())) k_zinv4(c
         sz[i] = from_f64<R>(sinz[i]);
     }
     __syncthreads();
-    const int ntx = (nxh + F4::W - 1) / F4::W;
-    for (int t = blockIdx.x; t < (ny + 2) * ntx; t += gridDim.x)
-        if (phi_only) zinv_tile_phi<R, NZ>(S, F, ny, nxh, ntx, t, tw, buf);
-        else zinv_tile<R, NZ>(S, F, ny, nxh, ntx, t, fstride, tw, sz, buf);
+    const int ncols = ny * nxh, fcols = (ny + 2) * nxh;
+    const int np = (ncols + F4::W - 1) / F4::W, ne = phi_only ? 0 : (fcols + F4::W - 1) / F4::W;
+    // the longer tiles (two transforms) first
+    for (int t = blockIdx.x; t < np + ne; t += gridDim.x) {
+        if (t >= np) zinv_tile_e<R, NZ>(F + fstride, fcols, t - np, tw, buf);
+        else if (phi_only) zinv_tile_phi<R, NZ, false>(S, F + nxh, ncols, fcols, t, fstride, tw, sz, buf);
+        else zinv_tile_phi<R, NZ, true>(S, F + nxh, ncols, fcols, t, fstride, tw, sz, buf);
+    }
 }
 
 // ---------------------------------------------------------------- x inverse
@@ -587,7 +603,7 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
                                                     double* __restrict__ phi, int ny, int nz, size_t fstride,
                                                     const double* __restrict__ sinx,
                                                     const cplx<R>* __restrict__ tw_g, int want_phi, int want_e,
-                                                    R norm, size_t nodes, const FastTab<R>* __restrict__ tab) {
+                                                    size_t nodes, const FastTab<R>* __restrict__ tab) {
     pdl_wait();
     if constexpr (kTab) {
         const FastTab<R>& t = tab[blockIdx.y];
@@ -617,6 +633,12 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
     const bool live = l < LPB && line < nz * nyn;
     const int jn = live ? line % nyn : 0;
     const bool interior = jn >= 1 && jn <= ny;
+    // the second step's threads are N1 a line, packed as in the forward transform
+    const int l2 = threadIdx.x / N1, r2 = threadIdx.x % N1;
+    const int line2 = tb * LPB + l2;
+    const bool live2 = l2 < LPB && line2 < nz * nyn;
+    const int jn2 = live2 ? line2 % nyn : 0;
+    const bool interior2 = jn2 >= 1 && jn2 <= ny;
     const int nf = want_phi ? 4 : 3;
     for (int f = want_e ? 0 : 3; f < nf; ++f) {
         const bool active = live && (f == 1 || interior);
@@ -627,15 +649,8 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
 #pragma unroll
             for (int n1 = 0; n1 < N1; ++n1) {
                 const int m = N2 * n1 + r;
-                cplx<R> xa = X[m], xb = X[M - m];
-                if (f == 0) {     // E_x multiplier -i sin(2 pi m / nx) / dx
-                    xa = cplx<R>{sx[m] * xa.im, -sx[m] * xa.re};
-                    xb = cplx<R>{sx[M - m] * xb.im, -sx[M - m] * xb.re};
-                }
-                const cplx<R> cb = conj(xb);
-                const cplx<R> sum = xa + cb;
-                const cplx<R> t = conj(tw[m]) * (xa - cb);
-                y[n1] = cplx<R>{sum.re - t.im, sum.im + t.re};
+                const cplx<R> xa = X[m], xb = X[M - m];
+                y[n1] = f == 0 ? split_inv_dx(xa, xb, tw[m], sx[m]) : split_inv(xa, xb, tw[m]);
             }
             fft::reg_dft<R, 1, N1, 2 * N2>(y, tw);
 #pragma unroll
@@ -645,26 +660,26 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
             for (int k1 = 0; k1 < N1; ++k1) b[k1] = y[k1];
         }
         __syncthreads();
-        if (active && r < N1) {
+        if (live2 && (f == 1 || interior2)) {
             cplx<R> z[N2];
-            const cplx<R>* b = buf + l * CS + r;
+            const cplx<R>* b = buf + l2 * CS + r2;
 #pragma unroll
             for (int n2 = 0; n2 < N2; ++n2) z[n2] = b[n2 * (N1 + 1)];
             fft::reg_dft<R, 1, N2, 2 * N1>(z, tw);
             if (f < 3) {
-                R* row = E + (size_t)f * nodes + (size_t)line * NX;
+                R* row = E + (size_t)f * nodes + (size_t)line2 * NX;
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
-                    const int k = r + N1 * k2;
-                    store_pair<R>(row + 2 * k, z[k2].re * norm, z[k2].im * norm);
+                    const int k = r2 + N1 * k2;
+                    store_pair<R>(row + 2 * k, z[k2].re, z[k2].im);
                 }
             } else {
-                double* prow = phi + ((size_t)(line / nyn) * ny + (jn - 1)) * NX;
+                double* prow = phi + ((size_t)(line2 / nyn) * ny + (jn2 - 1)) * NX;
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
-                    const int k = r + N1 * k2;
-                    prow[2 * k] = (double)(z[k2].re * norm);
-                    prow[2 * k + 1] = (double)(z[k2].im * norm);
+                    const int k = r2 + N1 * k2;
+                    prow[2 * k] = (double)z[k2].re;
+                    prow[2 * k + 1] = (double)z[k2].im;
                 }
             }
         }

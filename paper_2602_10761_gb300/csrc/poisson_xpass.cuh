@@ -29,22 +29,21 @@ void xinv_one(const PassGrid<R>& g, const cplx<R>* F, R* E, double* phi, const d
     constexpr int LPB = fft::FourStep<M, kThreads>::W;
     const int nlines = g.nz * (g.ny + 2);
     const size_t fstride = (size_t)g.nz * (g.ny + 2) * g.nxh, nodes = (size_t)nlines * g.nx;
-    const R norm = (R)(1.0 / ((double)g.nx * (double)g.nz));
     const int64_t tiles = (nlines + LPB - 1) / LPB;
     if constexpr (sizeof(R) == 4) {
         if (g.tab) {
             static int occ_tab = 0;
             const int gx = std::max(1, wave_blocks(k_xinv4<R, M, true>, xinv_smem<R, M>(), g.num_sms, tiles, &occ_tab) / g.n);
             k_xinv4<R, M, true><<<dim3(gx, g.n), kThreads, xinv_smem<R, M>(), g.stream>>>(
-                nullptr, nullptr, nullptr, g.ny, g.nz, fstride, nullptr, nullptr, 0, 1, norm, nodes, g.tab);
+                nullptr, nullptr, nullptr, g.ny, g.nz, fstride, nullptr, nullptr, 0, 1, nodes, g.tab);
             return;
         }
     }
     static int occ = 0;
     const int nb = wave_blocks(k_xinv4<R, M>, xinv_smem<R, M>(), g.num_sms, tiles, &occ);
     k_xinv4<R, M><<<nb, kThreads, xinv_smem<R, M>(), g.stream>>>(F, E, phi, g.ny, g.nz, fstride, sinx, twx,
-                                                                 phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, norm,
-                                                                 nodes, nullptr);
+                                                                 phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, nodes,
+                                                                 nullptr);
 }
 
 template <class R, int M>

@@ -11,7 +11,7 @@ namespace {
 template <class R, int NZ>
 void zfwd_one(const PassGrid<R>& g, cplx<R>* S, const cplx<R>* twz) {
     constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    const int64_t tiles = (int64_t)g.ny * ((g.nxh + W - 1) / W);
+    const int64_t tiles = ((int64_t)g.ny * g.nxh + W - 1) / W;
     if constexpr (sizeof(R) == 4) {
         if (g.tab) {
             static int occ_tab = 0;
@@ -31,7 +31,7 @@ template <class R, int NZ>
 void zinv_one(const PassGrid<R>& g, const cplx<R>* S, cplx<R>* F, const double* sinz, const cplx<R>* twz,
               bool phi_only) {
     constexpr int W = fft::FourStep<NZ, kThreads>::W;
-    const int64_t tiles = (int64_t)(g.ny + 2) * ((g.nxh + W - 1) / W);
+    const int64_t tiles = ((int64_t)g.ny * g.nxh + W - 1) / W + ((int64_t)(g.ny + 2) * g.nxh + W - 1) / W;
     const size_t fstride = (size_t)g.nz * (g.ny + 2) * g.nxh;
     if constexpr (sizeof(R) == 4) {
         if (g.tab) {

@@ -98,6 +98,16 @@ tribo_status check_params(const tribo_params* p) {
     return TRIBO_OK;
 }
 
+// per-row factors of the forward x transform: charge sums and densities to the right-hand side
+// -rho/eps, with the inverse transforms' normalisation
+void row_scales(const tribo_ctx* c, std::vector<double>& sq, std::vector<double>& sr) {
+    const double cells = (double)c->nx * (double)c->nz;
+    for (int j = 0; j < c->ny; ++j) {
+        sq[j] = -1.0 / (c->P.eps * c->dx * c->dy[j] * c->dz) / cells;
+        sr[j] = -1.0 / c->P.eps / cells;
+    }
+}
+
 tribo_status build_tables(tribo_ctx* c) {
     const int nx = c->nx, ny = c->ny, nz = c->nz;
     std::vector<float> xf(nx + 1), zf(nz + 1), yfu(ny + 1);
@@ -119,10 +129,7 @@ tribo_status build_tables(tribo_ctx* c) {
     }
     if ((st = upload(&c->d_ybin, bins))) return st;
     std::vector<double> sq(ny), sr(ny);
-    for (int j = 0; j < ny; ++j) {
-        sq[j] = -1.0 / (c->P.eps * c->dx * c->dy[j] * c->dz);
-        sr[j] = -1.0 / c->P.eps;
-    }
+    row_scales(c, sq, sr);
     if ((st = upload(&c->d_scale_q, sq)) || (st = upload(&c->d_scale_rho, sr))) return st;
     const size_t rs = real_size(c);
     std::vector<double> Yd = c->Y, inv(ny + 1);
@@ -611,10 +618,7 @@ tribo_status tribo_set_params(tribo_ctx* c, const tribo_params* params) {
     c->P = *params;
     if (eps_changed) {
         std::vector<double> sq(c->ny), sr(c->ny);
-        for (int j = 0; j < c->ny; ++j) {
-            sq[j] = -1.0 / (c->P.eps * c->dx * c->dy[j] * c->dz);
-            sr[j] = -1.0 / c->P.eps;
-        }
+        row_scales(c, sq, sr);
         TRIBO_CUDA(cudaStreamSynchronize(c->stream));
         TRIBO_CUDA(cudaMemcpy(c->d_scale_q, sq.data(), sizeof(double) * c->ny, cudaMemcpyHostToDevice));
         TRIBO_CUDA(cudaMemcpy(c->d_scale_rho, sr.data(), sizeof(double) * c->ny, cudaMemcpyHostToDevice));
