@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kThreads) k_pp_partner(PView p, const uint32_t
                                                          const uint32_t* __restrict__ offsets,
                                                          const uint32_t* __restrict__ members, uint32_t ncell,
                                                          uint32_t* __restrict__ partner) {
+    pdl_wait();
     const R* X = (const R*)p.x; const R* Y = (const R*)p.y; const R* Z = (const R*)p.z;
     const R* VX = (const R*)p.vx; const R* VY = (const R*)p.vy; const R* VZ = (const R*)p.vz;
     const R* D = (const R*)p.d;
@@ -77,6 +78,7 @@ template <class R>
 __global__ void __launch_bounds__(kThreads) k_pp_collide(PView p, const uint32_t* __restrict__ partner,
                                                          double rho_p, double k_e, double el, double eps,
                                                          double phi_p) {
+    pdl_wait();
     R* X = (R*)p.x; R* Y = (R*)p.y; R* Z = (R*)p.z;
     R* VX = (R*)p.vx; R* VY = (R*)p.vy; R* VZ = (R*)p.vz;
     const R* D = (const R*)p.d;
@@ -121,14 +123,13 @@ template <class R>
 tribo_status collide_impl(tribo_ctx* c, const PView& p, const uint32_t* members, uint32_t* partner) {
     const uint32_t ncell = (uint32_t)((size_t)c->nx * c->ny * c->nz);
     phase_begin(c, PH_AUX);
-    k_pp_partner<R><<<grid_for(p.n), kThreads, 0, c->stream>>>(p, c->sort_key, c->sort_counts, members, ncell,
-                                                               partner);
+    (void)launch_pdl(k_pp_partner<R>, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, p, (const uint32_t*)c->sort_key,
+                     (const uint32_t*)c->sort_counts, members, ncell, partner);
     TRIBO_LAUNCHED(c);
     const tribo_params& P = c->P;
     phase_begin(c, PH_AUX);
-    k_pp_collide<R><<<grid_for(p.n), kThreads, 0, c->stream>>>(p, partner, P.rho_p, P.k_e,
-                                                               2.0 * (1.0 - P.mu_p * P.mu_p) / P.E_p, P.eps,
-                                                               P.phi_p);
+    (void)launch_pdl(k_pp_collide<R>, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, p, (const uint32_t*)partner,
+                     P.rho_p, P.k_e, 2.0 * (1.0 - P.mu_p * P.mu_p) / P.E_p, P.eps, P.phi_p);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }

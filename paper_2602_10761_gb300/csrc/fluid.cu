@@ -29,6 +29,7 @@ template <class R>
 __global__ void k_mode_phase(int rows, int nm, const double* __restrict__ mf, const double* __restrict__ Y,
                              const double* __restrict__ ubar, const double* __restrict__ damp, double t,
                              cplx<R>* __restrict__ out) {
+    pdl_wait();
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)rows * nm) return;
     const int jn = (int)(idx / nm), m = (int)(idx - (int64_t)jn * nm);
@@ -54,6 +55,7 @@ __global__ void __launch_bounds__(kEvalThreads)
 k_mode_eval(int nx, int ny2, int nz, int nm, const int2* __restrict__ ma, const double* __restrict__ mf,
             const cplx<R>* __restrict__ mc, const cplx<R>* __restrict__ tabx, const cplx<R>* __restrict__ tabz,
             const double* __restrict__ ubar, R* __restrict__ out) {
+    pdl_wait();
     __shared__ cplx<R> G[kRows][kModeChunk];      // c_m(jn) Z_m(k) per row of the block
     __shared__ vec4<R> A[kModeChunk];             // amplitude vector
     __shared__ int AX[kModeChunk];                // nxi mod 2 nx
@@ -151,13 +153,14 @@ tribo_status eval_impl(tribo_ctx* c, double t, void* dst) {
     const int rows = c->ny + 2, nm = c->n_modes;
     const int64_t tot = (int64_t)rows * nm;
     phase_begin(c, PH_FIELD);
-    k_mode_phase<R><<<(unsigned)((tot + 255) / 256), 256, 0, c->stream>>>(
-        rows, nm, c->d_mode_f, c->d_Y, c->d_ubar, c->d_damp, t, (cplx<R>*)c->d_mode_c);
+    (void)launch_pdl(k_mode_phase<R>, dim3((unsigned)((tot + 255) / 256)), dim3(256), 0, c->stream, rows, nm,
+                     (const double*)c->d_mode_f, (const double*)c->d_Y, (const double*)c->d_ubar,
+                     (const double*)c->d_damp, t, (cplx<R>*)c->d_mode_c);
     TRIBO_LAUNCHED(c);
     phase_begin(c, PH_FIELD);
-    k_mode_eval<R><<<dim3((c->nz + kRows - 1) / kRows, rows), kEvalThreads, 0, c->stream>>>(
-        c->nx, rows, c->nz, nm, c->d_mode_a, c->d_mode_f, (const cplx<R>*)c->d_mode_c,
-        (const cplx<R>*)c->d_tabx, (const cplx<R>*)c->d_tabz, c->d_ubar, (R*)dst);
+    (void)launch_pdl(k_mode_eval<R>, dim3((c->nz + kRows - 1) / kRows, rows), dim3(kEvalThreads), 0, c->stream, c->nx,
+                     rows, c->nz, nm, (const int2*)c->d_mode_a, (const double*)c->d_mode_f, (const cplx<R>*)c->d_mode_c,
+                     (const cplx<R>*)c->d_tabx, (const cplx<R>*)c->d_tabz, (const double*)c->d_ubar, (R*)dst);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }

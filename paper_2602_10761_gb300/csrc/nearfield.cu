@@ -20,6 +20,7 @@ __global__ void __launch_bounds__(kThreads) k_coulomb(StepArgs<R> a, PView p, co
                                                       const uint32_t* __restrict__ offsets,
                                                       const uint32_t* __restrict__ members, uint32_t ncell,
                                                       double coef, R* __restrict__ acc) {
+    pdl_wait();
     const R* X = (const R*)p.x; const R* Y = (const R*)p.y; const R* Z = (const R*)p.z;
     const R* D = (const R*)p.d;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -54,8 +55,8 @@ tribo_status coulomb_impl(tribo_ctx* c, const PView& p, const uint32_t* members,
     StepArgs<R> a = make_args<R>(c, 0.0);
     const uint32_t ncell = (uint32_t)((size_t)c->nx * c->ny * c->nz);
     phase_begin(c, PH_AUX);
-    k_coulomb<R><<<grid_for(p.n), kThreads, 0, c->stream>>>(a, p, c->sort_key, c->sort_counts, members, ncell,
-                                                           1.0 / (4.0 * M_PI * c->P.eps), (R*)acoul);
+    (void)launch_pdl(k_coulomb<R>, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, a, p, (const uint32_t*)c->sort_key,
+                     (const uint32_t*)c->sort_counts, members, ncell, 1.0 / (4.0 * M_PI * c->P.eps), (R*)acoul);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }

@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(Ste
 
 template <class R>
 __global__ void k_deposit(StepArgs<R> a, PView p) {
+    pdl_wait();
     const R* X = (const R*)p.x; const R* Y = (const R*)p.y; const R* Z = (const R*)p.z;
     unsigned int err = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -80,6 +81,7 @@ __global__ void k_deposit(StepArgs<R> a, PView p) {
 }
 
 __global__ void k_sum_q(const double* __restrict__ q, int64_t n, double* out) {
+    pdl_wait();
     __shared__ double sh[kThreads / 32];
     double s = 0.0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -132,7 +134,7 @@ tribo_status deposit_impl(tribo_ctx* c, const PView& p) {
     StepArgs<R> a = make_args<R>(c, 0.0);
     a.Q = (double*)c->Q;
     phase_begin(c, PH_DEPOSIT);
-    k_deposit<R><<<grid_for(p.n), kThreads, 0, c->stream>>>(a, p);
+    (void)launch_pdl(k_deposit<R>, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, a, p);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }
@@ -146,6 +148,7 @@ tribo_status deposit_impl(tribo_ctx* c, const PView& p) {
 template <class R>
 __global__ void k_sort_count(StepArgs<R> a, PView p, uint32_t* __restrict__ counts, uint32_t* __restrict__ key,
                              uint32_t* __restrict__ rank) {
+    pdl_wait();
     const R* X = (const R*)p.x; const R* Y = (const R*)p.y; const R* Z = (const R*)p.z;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; n < p.n; n += stride) {
@@ -163,6 +166,7 @@ __global__ void k_sort_count(StepArgs<R> a, PView p, uint32_t* __restrict__ coun
 // nearly so (the particles move little between sorts)
 template <class R>
 __global__ void k_sort_gather(PView src, PView dst, const uint32_t* __restrict__ perm) {
+    pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; d < src.n; d += stride) {
         const uint32_t n = perm[d];
@@ -205,6 +209,7 @@ __device__ __forceinline__ void store4(void* dst, int64_t t, const Four<T>& f) {
 
 template <class R>
 __global__ void k_sort_gather4(PView src, PView dst, const uint32_t* __restrict__ perm) {
+    pdl_wait();
     const int64_t n4 = src.n / 4;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n4; t += stride) {
@@ -287,6 +292,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* s
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t* __restrict__ in, size_t n,
                                                              uint32_t* __restrict__ tile_sums) {
+    pdl_wait();
     __shared__ uint32_t sh[32];
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanPer;
     uint32_t s = 0;
@@ -304,6 +310,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t* __r
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* __restrict__ sums, int nt) {
+    pdl_wait();
     __shared__ uint32_t sh[32];
     __shared__ uint32_t carry;
     if (threadIdx.x == 0) carry = 0;
@@ -322,6 +329,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_sums(uint32_t* __restrict
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(uint32_t* __restrict__ data, size_t n,
                                                              const uint32_t* __restrict__ tile_off) {
+    pdl_wait();
     __shared__ uint32_t sh[32];
     const size_t base = (size_t)blockIdx.x * kScanTile + (size_t)threadIdx.x * kScanPer;
     uint32_t v[kScanPer];
@@ -358,6 +366,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(uint32_t* __restric
 
 __global__ void k_cell_members(const uint32_t* __restrict__ offsets, const uint32_t* __restrict__ key,
                                const uint32_t* __restrict__ rank, int64_t n, uint32_t* __restrict__ members) {
+    pdl_wait();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
         members[offsets[key[i]] + rank[i]] = (uint32_t)i;
@@ -366,59 +375,41 @@ __global__ void k_cell_members(const uint32_t* __restrict__ offsets, const uint3
 // per-cell lists: key and rank of every particle, cell offsets (exclusive
 // scan of the counts) in sort_counts, members grouped by cell
 template <class R>
-tribo_status cell_lists_impl(tribo_ctx* c, const PView& p, uint32_t* members) {
+tribo_status cell_lists_impl(tribo_ctx* c, const PView& p, uint32_t* members, int phase) {
     const size_t ncell = (size_t)c->nx * c->ny * c->nz;
     const int ntiles = (int)((ncell + kScanTile - 1) / kScanTile);
-    phase_begin(c, PH_AUX);
+    phase_begin(c, phase);
     TRIBO_CUDA(cudaMemsetAsync(c->sort_counts, 0, sizeof(uint32_t) * ncell, c->stream));
     StepArgs<R> a = make_args<R>(c, 0.0);
-    k_sort_count<R><<<grid_for(p.n), kThreads, 0, c->stream>>>(a, p, c->sort_counts, c->sort_key, c->sort_rank);
+    (void)launch_pdl(k_sort_count<R>, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, a, p, c->sort_counts,
+                     c->sort_key, c->sort_rank);
     TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_AUX);
-    k_scan_tiles<<<ntiles, kScanThreads, 0, c->stream>>>(c->sort_counts, ncell, c->sort_tiles);
+    phase_begin(c, phase);
+    (void)launch_pdl(k_scan_tiles, dim3(ntiles), dim3(kScanThreads), 0, c->stream, (const uint32_t*)c->sort_counts,
+                     ncell, c->sort_tiles);
     TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_AUX);
-    k_scan_sums<<<1, kScanThreads, 0, c->stream>>>(c->sort_tiles, ntiles);
+    phase_begin(c, phase);
+    (void)launch_pdl(k_scan_sums, dim3(1), dim3(kScanThreads), 0, c->stream, c->sort_tiles, ntiles);
     TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_AUX);
-    k_scan_apply<<<ntiles, kScanThreads, 0, c->stream>>>(c->sort_counts, ncell, c->sort_tiles);
+    phase_begin(c, phase);
+    (void)launch_pdl(k_scan_apply, dim3(ntiles), dim3(kScanThreads), 0, c->stream, c->sort_counts, ncell,
+                     (const uint32_t*)c->sort_tiles);
     TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_AUX);
-    k_cell_members<<<grid_for(p.n), kThreads, 0, c->stream>>>(c->sort_counts, c->sort_key, c->sort_rank, p.n,
-                                                              members);
+    phase_begin(c, phase);
+    (void)launch_pdl(k_cell_members, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, (const uint32_t*)c->sort_counts,
+                     (const uint32_t*)c->sort_key, (const uint32_t*)c->sort_rank, p.n, members);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }
 
 template <class R>
 tribo_status sort_impl(tribo_ctx* c, const PView& src, const PView& dst) {
-    const size_t ncell = (size_t)c->nx * c->ny * c->nz;
-    uint32_t* counts = c->sort_counts;
-    uint32_t* key = c->sort_key;
-    uint32_t* rank = c->sort_rank;
-    const int ntiles = (int)((ncell + kScanTile - 1) / kScanTile);
+    tribo_status st = cell_lists_impl<R>(c, src, c->sort_perm, PH_SORT);
+    if (st) return st;
     phase_begin(c, PH_SORT);
-    TRIBO_CUDA(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * ncell, c->stream));
-    StepArgs<R> a = make_args<R>(c, 0.0);
-    k_sort_count<R><<<grid_for(src.n), kThreads, 0, c->stream>>>(a, src, counts, key, rank);
-    TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_SORT);
-    k_scan_tiles<<<ntiles, kScanThreads, 0, c->stream>>>(counts, ncell, c->sort_tiles);
-    TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_SORT);
-    k_scan_sums<<<1, kScanThreads, 0, c->stream>>>(c->sort_tiles, ntiles);
-    TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_SORT);
-    k_scan_apply<<<ntiles, kScanThreads, 0, c->stream>>>(counts, ncell, c->sort_tiles);
-    TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_SORT);
-    k_cell_members<<<grid_for(src.n), kThreads, 0, c->stream>>>(counts, key, rank, src.n, c->sort_perm);
-    TRIBO_LAUNCHED(c);
-    phase_begin(c, PH_SORT);
-    if (gather4_ok(src, dst))
-        k_sort_gather4<R><<<grid_for((src.n + 3) / 4), kThreads, 0, c->stream>>>(src, dst, c->sort_perm);
-    else
-        k_sort_gather<R><<<grid_for(src.n), kThreads, 0, c->stream>>>(src, dst, c->sort_perm);
+    const bool four = gather4_ok(src, dst);
+    (void)launch_pdl(four ? k_sort_gather4<R> : k_sort_gather<R>, dim3(grid_for(four ? (src.n + 3) / 4 : src.n)),
+                     dim3(kThreads), 0, c->stream, src, dst, (const uint32_t*)c->sort_perm);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }
@@ -433,8 +424,8 @@ tribo_status particles_sort(tribo_ctx* c, const PView& src, const PView& dst) {
 
 tribo_status particles_cell_lists(tribo_ctx* c, const PView& p, uint32_t* members) {
     if (p.n == 0) return TRIBO_OK;
-    if (c->prec == TRIBO_FP64) return cell_lists_impl<double>(c, p, members);
-    return cell_lists_impl<float>(c, p, members);
+    if (c->prec == TRIBO_FP64) return cell_lists_impl<double>(c, p, members, PH_AUX);
+    return cell_lists_impl<float>(c, p, members, PH_AUX);
 }
 
 tribo_status particles_step(tribo_ctx* c, const PView& p, double dt, bool deposit_next, bool write_cell,
@@ -454,7 +445,7 @@ tribo_status particles_sum_q(tribo_ctx* c, const PView& p, double* d_out) {
     TRIBO_CUDA(cudaMemsetAsync(d_out, 0, sizeof(double), c->stream));
     if (p.n == 0) return TRIBO_OK;
     phase_begin(c, PH_AUX);
-    k_sum_q<<<grid_for(p.n), kThreads, 0, c->stream>>>(p.q, p.n, d_out);
+    (void)launch_pdl(k_sum_q, dim3(grid_for(p.n)), dim3(kThreads), 0, c->stream, (const double*)p.q, p.n, d_out);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }

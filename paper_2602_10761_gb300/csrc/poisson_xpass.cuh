@@ -41,9 +41,8 @@ void xinv_one(const PassGrid<R>& g, const cplx<R>* F, R* E, double* phi, const d
     }
     static int occ = 0;
     const int nb = wave_blocks(k_xinv4<R, M>, xinv_smem<R, M>(), g.num_sms, tiles, &occ);
-    k_xinv4<R, M><<<nb, kThreads, xinv_smem<R, M>(), g.stream>>>(F, E, phi, g.ny, g.nz, fstride, sinx, twx,
-                                                                 phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, nodes,
-                                                                 nullptr);
+    (void)launch_pdl(k_xinv4<R, M>, dim3(nb), dim3(kThreads), xinv_smem<R, M>(), g.stream, F, E, phi, g.ny, g.nz, fstride,
+                     sinx, twx, phi != nullptr ? 1 : 0, E != nullptr ? 1 : 0, nodes, (const FastTab<R>*)nullptr);
 }
 
 template <class R, int M>

@@ -44,8 +44,8 @@ void zinv_one(const PassGrid<R>& g, const cplx<R>* S, cplx<R>* F, const double* 
     }
     static int occ = 0;
     const int nb = wave_blocks(k_zinv4<R, NZ>, zinv_smem<R, NZ>(), g.num_sms, tiles, &occ);
-    k_zinv4<R, NZ><<<nb, kThreads, zinv_smem<R, NZ>(), g.stream>>>(S, F, g.ny, g.nxh, fstride, sinz, twz,
-                                                                   phi_only ? 1 : 0, nullptr);
+    (void)launch_pdl(k_zinv4<R, NZ>, dim3(nb), dim3(kThreads), zinv_smem<R, NZ>(), g.stream, S, F, g.ny, g.nxh, fstride,
+                     sinz, twz, phi_only ? 1 : 0, (const FastTab<R>*)nullptr);
 }
 
 template <class R, int NZ>
