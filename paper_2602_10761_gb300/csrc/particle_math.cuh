@@ -355,17 +355,38 @@ __device__ __forceinline__ void phi12(double s, double& phi1, double& phi2) {
     }
 }
 
-// the condenser-model charge of one wall impact (FP64)
+// x^(2/5), x > 0, in FP64: a particle that meets a wall holds its warp for the length of this chain,
+// so it is kept short.  y0 = x^(2/5) to FP32 accuracy; with e = x^2 / y0^5 - 1 (about 1e-6),
+// x^(2/5) = y0 (1 + e)^(1/5) = y0 (1 + e/5 - 2 e^2/25 + O(e^3)), the cube below 1e-17.
+__device__ __forceinline__ double pow04(double x) {
+    if (!(x > 1e-30 && x < 1e30)) return pow(x, 0.4);
+    const double y = (double)exp2f(0.4f * log2f((float)x));
+    const double y2 = y * y;
+    const double e = x * x / (y2 * y2 * y) - 1.0;
+    return y + y * (e * (0.2 - 0.08 * e));
+}
+// 1 - e^-x, x >= 0
+__device__ __forceinline__ double one_minus_exp(double x) {
+    if (x < 0.5) {
+        double p1, p2;
+        phi12(x, p1, p2);
+        return p1;
+    }
+    return -expm1(-x);
+}
+
+// the condenser-model charge of one wall impact (FP64) at the squared speed s2: with P = (alpha_coef
+// s2)^(2/5), alpha = r P and A = kappa_pi r alpha, so that A / (pi d^2) = kappa_pi P / (4 pi)
 template <class R>
-__device__ __forceinline__ double impact_charge(const StepArgs<R>& a, double d, double speed, double q) {
-    if (!(speed > 0.0)) return 0.0;
+__device__ __forceinline__ double impact_charge(const StepArgs<R>& a, double d, double s2, double q) {
+    if (!(s2 > 0.0)) return 0.0;
     const double r = 0.5 * d;
-    const double alpha = r * pow(a.alpha_coef * speed * speed, 0.4);
-    const double A = a.kappa_pi * r * alpha;
-    const double C = a.eps_over_h * A;
-    const double dt_w = 2.94 * alpha / speed;
-    double dq = -C * a.U_c * (-expm1(-dt_w * a.inv_T_w));
-    if (a.dq_t) dq += -(A / (M_PI * d * d)) * q;
+    const double P = pow04(a.alpha_coef * s2);
+    const double alpha = r * P;
+    const double C = a.eps_over_h * (a.kappa_pi * r * alpha);
+    const double dt_w = 2.94 * alpha * rsqrt(s2);
+    double dq = -C * a.U_c * one_minus_exp(dt_w * a.inv_T_w);
+    if (a.dq_t) dq += -(a.kappa_pi * (0.25 / M_PI) * P) * q;
     return dq;
 }
 
@@ -392,10 +413,10 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 // (q the charge before the impact, q_max = sgn(dq0_min) c_sat d^2 / 4, so
 // q / q_max = sgn(dq0_min) 4 q / (c_sat d^2))
 template <class R>
-__device__ __noinline__ double ssm_charge(const StepArgs<R>& a, double d, double speed, double q, unsigned int id,
+__device__ __noinline__ double ssm_charge(const StepArgs<R>& a, double d, double s2, double q, unsigned int id,
                                           unsigned int count, double* site) {
     const double r = 0.5 * d;
-    const double A = M_PI * r * r * pow(a.alpha_coef * speed * speed, 0.4);
+    const double A = M_PI * r * r * pow04(a.alpha_coef * s2);
     const double area = A * a.ssm_inv_A0;
     const double x = a.ssm_xcoef * q / (d * d);
     const double sw = a.ssm_dq0min > 0.0 ? 1.0 : (a.ssm_dq0min < 0.0 ? -1.0 : 0.0);
@@ -413,8 +434,8 @@ __device__ __noinline__ double ssm_charge(const StepArgs<R>& a, double d, double
     g = fmin(fmax(g, -0.99), 0.99);               // inside the family's range, well conditioned
     // skew-normal (xi, omega, delta) from the mean, deviation and skewness
     const double b = 0.7978845608028654;          // sqrt(2 / pi)
-    const double ag = pow(fabs(g), 2.0 / 3.0);
-    const double t = ag / (pow(0.5 * (4.0 - M_PI), 2.0 / 3.0) + ag);
+    const double ag = cbrt(g * g);                // |g|^(2/3)
+    const double t = ag / (0.5689956594119245 + ag);   // ((4 - pi) / 2)^(2/3)
     const double delta = (g > 0.0 ? 1.0 : (g < 0.0 ? -1.0 : 0.0)) * sqrt(t) / b;
     const double omega = sigma_i / sqrt(1.0 - 2.0 * delta * delta / M_PI);
     const double xi = mu_i - omega * delta * b;
@@ -488,10 +509,13 @@ int grid_for(int64_t n, int threads = kThreads) {
 }
 
 // one particle of the coupled step (the body of k_step): gather, push,
-// wrap, wall impact with the condenser charge, deposit for the next step
-template <class R>
+// wrap, wall impact with the condenser charge, deposit for the next step.  kOut: the new positions,
+// velocities and charges go to `o` (the adjoint's stored states) and p keeps the old ones; the wall
+// charge and the impact count are p's either way.
+template <class R, bool kOut = false>
 __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, int64_t n, int write_cell,
-                                         unsigned int* sh_hist, bool use_hist, unsigned int& err) {
+                                         unsigned int* sh_hist, bool use_hist, unsigned int& err,
+                                         const PView* o = nullptr) {
     R* X = (R*)p.x; R* Y = (R*)p.y; R* Z = (R*)p.z;
     R* VX = (R*)p.vx; R* VY = (R*)p.vy; R* VZ = (R*)p.vz;
     const R* D = (const R*)p.d;
@@ -596,22 +620,19 @@ __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, i
         yn = (R)ym;
         vyn = -vyn;
         if (yn < r || yn > a.ly - r) err |= TRIBO_DEV_ESCAPED;
-        double speed;
-        if (a.impact_vel == TRIBO_IMPACT_NORMAL) {
-            speed = fabs((double)vyn);
-        } else {
-            speed = sqrt((double)vxn * (double)vxn + (double)vyn * (double)vyn + (double)vzn * (double)vzn);
-        }
+        double s2 = (double)vyn * (double)vyn;          // squared impact speed
+        if (a.impact_vel != TRIBO_IMPACT_NORMAL)
+            s2 = (double)vxn * (double)vxn + s2 + (double)vzn * (double)vzn;
         double dq;
-        if (a.ssm && speed > 0.0) {
+        if (a.ssm && s2 > 0.0) {
             double site = p.site ? p.site[n] : 1.0;
-            dq = ssm_charge<R>(a, (double)d, speed, q, p.id[n], p.n_imp[n], &site);
+            dq = ssm_charge<R>(a, (double)d, s2, q, p.id[n], p.n_imp[n], &site);
             if (p.site) p.site[n] = site;
         } else {
-            dq = impact_charge<R>(a, (double)d, speed, q);
+            dq = impact_charge<R>(a, (double)d, s2, q);
         }
         q += dq;
-        p.q[n] = q;
+        if constexpr (!kOut) p.q[n] = q;
         p.q_wall[n] += dq;
         p.n_imp[n] += 1u;
         atomicAdd(&a.acc->sum_wall, dq);
@@ -619,8 +640,14 @@ __device__ __forceinline__ void step_one(const StepArgs<R>& a, const PView& p, i
     }
     if (!(step_finite(xn) && step_finite(yn) && step_finite(zn) && step_finite(vxn) && step_finite(vyn) && step_finite(vzn)))
         err |= TRIBO_DEV_NONFINITE;
-    X[n] = xn; Y[n] = yn; Z[n] = zn;
-    VX[n] = vxn; VY[n] = vyn; VZ[n] = vzn;
+    if constexpr (kOut) {
+        ((R*)o->x)[n] = xn; ((R*)o->y)[n] = yn; ((R*)o->z)[n] = zn;
+        ((R*)o->vx)[n] = vxn; ((R*)o->vy)[n] = vyn; ((R*)o->vz)[n] = vzn;
+        o->q[n] = q;
+    } else {
+        X[n] = xn; Y[n] = yn; Z[n] = zn;
+        VX[n] = vxn; VY[n] = vyn; VZ[n] = vzn;
+    }
     int jn;
     const uint32_t key = cell_key_near<R>(xn, yn, zn, a, j, &jn, rows ? &yr : nullptr);
     if (a.Q) atomicAdd(&a.Q[key], q);
