@@ -24,9 +24,12 @@
 //                so Q-bar = L^-1 (scale * phi-bar): the same solve as the
 //                forward field, with the same per-row scale.
 //   k_adj_deposit  q-bar_p += Q-bar[cell(x_p)] (transpose of the deposit).
-// Forward states are kept every ckpt_every steps; each segment is recomputed
-// from its checkpoint (states and field lattices of the segment stored) before
-// it is reversed.
+// The state and the field of every forward step are kept in HBM when they fit in
+// the budget; the reverse sweep then reads them.  Otherwise states are kept every
+// ckpt_every steps and each segment is recomputed from its checkpoint (states and
+// field lattices of the segment stored) before it is reversed.  Each stored state
+// is written by the step itself (k_step's kOut form), not copied.  128^3, 1M
+// particles, 12 steps, a checkpoint every 4: 5.0 -> 4.24 ms with the states kept.
 #include <cmath>
 #include <cstdio>
 #include <vector>
@@ -434,12 +437,11 @@ template <class R>
 struct AdjLayout {
     std::vector<SView<R>> ckpt, seg;
     std::vector<R*> segE;
-    SView<R> W, lam;
+    SView<R> lam;
     double* Wqw;
     uint32_t* Wni;
     R* Eb;
     double* psi;
-    R* cy;
     double* pacc;
     double* db;
     Accum* acc;
@@ -451,23 +453,21 @@ constexpr size_t eb_reals() { return sizeof(R) == 4 ? 4 : 3; }
 
 // carve the workspace (base NULL: only count the bytes)
 template <class R>
-size_t layout(AdjLayout<R>& L, char* base, int64_t n, int nseg, int C, bool electro, size_t nodes, size_t ncell,
-              int ny) {
+size_t layout(AdjLayout<R>& L, char* base, int64_t n, int nseg, int C, bool segfields, bool electro, size_t nodes,
+              size_t ncell) {
     Carve cv{base};
     L.ckpt.resize(nseg);
     for (int g = 0; g < nseg; ++g) L.ckpt[g] = take_state<R>(cv, n);
     L.seg.resize(C);
     for (int i = 0; i < C; ++i) L.seg[i] = take_state<R>(cv, n);
     L.segE.assign(C, nullptr);
-    if (electro)
+    if (segfields)
         for (int i = 0; i < C; ++i) L.segE[i] = (R*)cv.take(3 * nodes * sizeof(R));
-    L.W = take_state<R>(cv, n);
     L.Wqw = (double*)cv.take(n * sizeof(double));
     L.Wni = (uint32_t*)cv.take(n * sizeof(uint32_t));
     L.lam = take_state<R>(cv, n);
     L.Eb = electro ? (R*)cv.take(eb_reals<R>() * nodes * sizeof(R)) : nullptr;
     L.psi = electro ? (double*)cv.take(ncell * sizeof(double)) : nullptr;
-    L.cy = (R*)cv.take(3 * (size_t)ny * sizeof(R));
     L.pacc = (double*)cv.take(2 * sizeof(double));
     L.db = (double*)cv.take(n * sizeof(double));
     L.acc = (Accum*)cv.take(sizeof(Accum));
@@ -524,22 +524,71 @@ tribo_status adjoint_impl(tribo_ctx* c, const PView& P, double dt, int nsteps, i
     const int Cs = nsteps > 0 ? std::min(C, nsteps) : 0;
     const size_t nodes = (size_t)c->nz * (c->ny + 2) * c->nx;
     const size_t ncell = (size_t)c->nx * c->ny * c->nz;
+    // the fields and the states of all forward steps, kept when they fit in the budget (half of the
+    // free memory by default): with both, nothing is recomputed; with the fields alone, the
+    // recomputed segments take them instead of depositing and solving again
+    Carve one{nullptr};
+    take_state<R>(one, n);
+    const size_t ebytes = electro ? (3 * nodes * sizeof(R) + 255) & ~(size_t)255 : 0, sbytes = one.off;
+    bool keepE = false, keepS = false;
     AdjLayout<R> L;
-    const size_t bytes = layout<R>(L, nullptr, n, nseg, Cs, electro, nodes, ncell, c->ny);
-    if (bytes > c->adj_bytes) {
-        TRIBO_CUDA(cudaStreamSynchronize(c->stream));
-        if (c->adj) cudaFree(c->adj);
-        c->adj = nullptr;
-        c->adj_bytes = 0;
-        TRIBO_CUDA(cudaMalloc(&c->adj, bytes));
-        c->adj_bytes = bytes;
+    auto lay = [&](char* base) {
+        return layout<R>(L, base, n, keepS ? 0 : nseg, keepS ? 0 : Cs, electro && !keepE, electro, nodes, ncell);
+    };
+    for (int keep = nsteps > 0 ? 2 : 0;; --keep) {       // 2: fields and states, 1: fields, 0: neither
+        if (keep == 1 && !electro) continue;
+        keepE = keep >= 1 && electro;
+        keepS = keep == 2;
+        const size_t need = ((keepE ? ebytes : 0) + (keepS ? sbytes : 0)) * (size_t)nsteps;
+        const size_t bytes = lay(nullptr), grow = bytes > c->adj_bytes ? bytes : 0;
+        if (c->adj_E_limit >= 0) {
+            if (need > (size_t)c->adj_E_limit) continue;
+        } else if (need > c->adj_E_bytes) {
+            // half of what the workspace leaves free
+            size_t freeb = 0, total = 0;
+            if (cudaMemGetInfo(&freeb, &total) != cudaSuccess || freeb < grow || need > (freeb - grow) / 2) continue;
+        }
+        if (grow) {
+            TRIBO_CUDA(cudaStreamSynchronize(c->stream));
+            if (c->adj) cudaFree(c->adj);
+            c->adj = nullptr;
+            c->adj_bytes = 0;
+            const cudaError_t e = cudaMalloc(&c->adj, bytes);
+            if (e == cudaSuccess) {
+                c->adj_bytes = bytes;
+            } else if (keep > 0) {
+                (void)cudaGetLastError();
+                continue;
+            } else {
+                return cuda_fail(e, "adjoint workspace");
+            }
+        }
+        if (need > c->adj_E_bytes) {
+            TRIBO_CUDA(cudaStreamSynchronize(c->stream));
+            if (c->adj_E) cudaFree(c->adj_E);
+            c->adj_E = nullptr;
+            c->adj_E_bytes = 0;
+            if (cudaMalloc(&c->adj_E, need) != cudaSuccess) {
+                (void)cudaGetLastError();
+                continue;
+            }
+            c->adj_E_bytes = need;
+        }
+        break;
     }
-    layout<R>(L, (char*)c->adj, n, nseg, Cs, electro, nodes, ncell, c->ny);
+    lay((char*)c->adj);
+    auto E_of_step = [&](int s) -> R* { return (R*)((char*)c->adj_E + ebytes * (size_t)s); };
+    auto state_of_step = [&](int s) -> SView<R> {
+        Carve cv{(char*)c->adj_E + (keepE ? ebytes * (size_t)nsteps : 0) + sbytes * (size_t)s};
+        return take_state<R>(cv, n);
+    };
     double* db = dd ? dd : L.db;
-    const std::vector<double> cy64 = grad_transpose_y(c);
-    const std::vector<R> cy(cy64.begin(), cy64.end());
-    TRIBO_CUDA(cudaStreamSynchronize(c->stream));
-    TRIBO_CUDA(cudaMemcpy(L.cy, cy.data(), sizeof(R) * cy.size(), cudaMemcpyHostToDevice));
+    if (!c->adj_cy) {
+        const std::vector<double> cy64 = grad_transpose_y(c);
+        const std::vector<R> cy(cy64.begin(), cy64.end());
+        TRIBO_CUDA(cudaMalloc(&c->adj_cy, sizeof(R) * cy.size()));
+        TRIBO_CUDA(cudaMemcpy(c->adj_cy, cy.data(), sizeof(R) * cy.size(), cudaMemcpyHostToDevice));
+    }
     TRIBO_CUDA(cudaMemsetAsync(db, 0, n * sizeof(double), c->stream));
     TRIBO_CUDA(cudaMemsetAsync(L.pacc, 0, 2 * sizeof(double), c->stream));
     TRIBO_CUDA(cudaMemsetAsync(L.acc, 0, sizeof(Accum), c->stream));
@@ -547,43 +596,21 @@ tribo_status adjoint_impl(tribo_ctx* c, const PView& P, double dt, int nsteps, i
     const double t_start = c->time;
     const size_t qbytes = ncell * sizeof(double);   // the deposit's FP64 cell charge sums
 
-    // the field of every forward step kept in HBM when it fits in half of the free memory: the
-    // recomputed segments then take it instead of depositing and solving again
-    const size_t ebytes = 3 * nodes * sizeof(R);
-    bool keepE = false;
-    if (electro && nsteps > 0) {
-        const size_t need = ebytes * (size_t)nsteps;
-        if (c->adj_E_limit >= 0 && need > (size_t)c->adj_E_limit) {
-            keepE = false;
-        } else if (need <= c->adj_E_bytes) {
-            keepE = true;
-        } else {
-            size_t freeb = 0, total = 0;
-            const bool room = c->adj_E_limit >= 0 ||
-                              (cudaMemGetInfo(&freeb, &total) == cudaSuccess && need + c->adj_E_bytes <= freeb / 2);
-            if (room) {
-                TRIBO_CUDA(cudaStreamSynchronize(c->stream));
-                if (c->adj_E) cudaFree(c->adj_E);
-                c->adj_E = nullptr;
-                c->adj_E_bytes = 0;
-                if (cudaMalloc(&c->adj_E, need) == cudaSuccess) {
-                    c->adj_E_bytes = need;
-                    keepE = true;
-                } else {
-                    (void)cudaGetLastError();
-                }
-            }
-        }
-    }
-    auto E_of_step = [&](int s) -> R* { return (R*)((char*)c->adj_E + ebytes * (size_t)s); };
-
     // ---- forward pass on the caller's particles, with checkpoints
     if (electro && nsteps > 0) {
         TRIBO_CUDA(cudaMemsetAsync(c->Q, 0, qbytes, c->stream));
         if ((st = particles_deposit(c, P))) return st;
     }
+    // keeping the states: step s reads state s and writes state s + 1, the last one the caller's
+    // arrays again (the diameters, wall charges and impact counts are the caller's throughout)
+    auto as_particles = [&](const SView<R>& v) {
+        PView p = P;
+        p.x = v.x; p.y = v.y; p.z = v.z; p.vx = v.vx; p.vy = v.vy; p.vz = v.vz; p.q = v.q;
+        return p;
+    };
+    if (keepS && (st = copy_state<R>(c, state_of_step(0), state_of<R>(P), n))) return st;
     for (int s = 0; s < nsteps; ++s) {
-        if (s % C == 0 && (st = copy_state<R>(c, L.ckpt[s / C], state_of<R>(P), n))) return st;
+        if (!keepS && s % C == 0 && (st = copy_state<R>(c, L.ckpt[s / C], state_of<R>(P), n))) return st;
         if (c->n_modes && (st = modes_eval(c, t_start + s * dt, c->u_lat))) return st;
         StepIO fio;
         if (electro) {
@@ -591,7 +618,13 @@ tribo_status adjoint_impl(tribo_ctx* c, const PView& P, double dt, int nsteps, i
             if ((st = poisson_solve(c, c->Q, true, c->d_scale_q, true, nullptr, Es))) return st;
             fio.E = Es;
         }
-        if ((st = particles_step(c, P, dt, electro && s < nsteps - 1, P.cell != nullptr && s == nsteps - 1, fio)))
+        PView cur = P, out = P;
+        if (keepS) {
+            cur = as_particles(state_of_step(s));
+            if (s < nsteps - 1) out = as_particles(state_of_step(s + 1));
+            fio.out = &out;
+        }
+        if ((st = particles_step(c, cur, dt, electro && s < nsteps - 1, P.cell != nullptr && s == nsteps - 1, fio)))
             return st;
         c->steps_done++;
     }
@@ -609,39 +642,43 @@ tribo_status adjoint_impl(tribo_ctx* c, const PView& P, double dt, int nsteps, i
     // the field adjoint starts zero; each step's k_adj_deposit leaves it zero again
     const size_t eb_bytes = eb_reals<R>() * nodes * sizeof(R);
     if (electro) TRIBO_CUDA(cudaMemsetAsync(L.Eb, 0, eb_bytes, c->stream));
-    PView Wp{};
-    Wp.n = n;
-    Wp.x = L.W.x; Wp.y = L.W.y; Wp.z = L.W.z; Wp.vx = L.W.vx; Wp.vy = L.W.vy; Wp.vz = L.W.vz;
-    Wp.d = P.d; Wp.q = L.W.q; Wp.q_wall = L.Wqw; Wp.n_imp = L.Wni;
     StepIO io;
     io.acc = L.acc;
     io.stats = false;
     for (int g = nseg - 1; g >= 0; --g) {
         const int s0 = g * C;
         const int len = std::min(C, nsteps - s0);
-        if ((st = copy_state<R>(c, L.W, L.ckpt[g], n))) return st;
-        // the field of step s0 + i: kept from the forward pass, or solved again from the
-        // recomputed charges
+        // the field and the state of step s0 + i: kept from the forward pass, or recomputed
         auto segE = [&](int i) -> R* { return keepE ? E_of_step(s0 + i) : L.segE[i]; };
+        auto segS = [&](int i) -> SView<R> { return keepS ? state_of_step(s0 + i) : i == 0 ? L.ckpt[g] : L.seg[i]; };
+        auto recomputed = [&](const SView<R>& v) {          // with scratch wall charges and impact counts
+            PView p = as_particles(v);
+            p.q_wall = L.Wqw;
+            p.n_imp = L.Wni;
+            p.id = p.cell = nullptr;
+            return p;
+        };
         if (electro && !keepE) {
             TRIBO_CUDA(cudaMemsetAsync(c->Q, 0, qbytes, c->stream));
-            if ((st = particles_deposit(c, Wp))) return st;
+            if ((st = particles_deposit(c, recomputed(segS(0))))) return st;
         }
         for (int i = 0; i < len; ++i) {
-            if ((st = copy_state<R>(c, L.seg[i], L.W, n))) return st;
-            if (c->n_modes && (st = modes_eval(c, t_start + (s0 + i) * dt, c->u_lat))) return st;
+            if (c->n_modes && (!keepS || i == len - 1) && (st = modes_eval(c, t_start + (s0 + i) * dt, c->u_lat)))
+                return st;
             if (electro && !keepE && (st = poisson_solve(c, c->Q, true, c->d_scale_q, true, nullptr, L.segE[i])))
                 return st;
-            if (i < len - 1) {
+            if (i < len - 1 && !keepS) {
+                const PView out = recomputed(segS(i + 1));
                 io.E = electro ? (const void*)segE(i) : nullptr;
-                if ((st = particles_step(c, Wp, dt, electro && !keepE, false, io))) return st;
+                io.out = &out;
+                if ((st = particles_step(c, recomputed(segS(i)), dt, electro && !keepE, false, io))) return st;
             }
         }
         for (int i = len - 1; i >= 0; --i) {
             if (c->n_modes && i < len - 1 && (st = modes_eval(c, t_start + (s0 + i) * dt, c->u_lat))) return st;
             StepArgs<R> a = make_args<R>(c, dt);
             if (electro) a.E = segE(i);
-            AdjArgs<R> ga{L.seg[i], (const R*)P.d, L.lam, db, L.Eb, L.pacc, n, c->P.kappa_A};
+            AdjArgs<R> ga{segS(i), (const R*)P.d, L.lam, db, L.Eb, L.pacc, n, c->P.kappa_A};
             phase_begin(c, PH_ADJOINT);
             // one resident wave (two blocks per SM), as for the forward step
             const int ab = (int)std::min<int64_t>((n + kThreads - 1) / kThreads, (int64_t)c->num_sms * 2);
@@ -650,12 +687,12 @@ tribo_status adjoint_impl(tribo_ctx* c, const PView& P, double dt, int nsteps, i
             if (!electro) continue;
             const int gb = (int)std::min<int64_t>((int64_t)c->nz * c->ny, (int64_t)c->num_sms * 16);
             phase_begin(c, PH_ADJOINT);
-            (void)launch_pdl(k_adj_grad<R>, dim3(gb), dim3(128), 0, c->stream, (const R*)L.Eb, (const R*)L.cy,
+            (void)launch_pdl(k_adj_grad<R>, dim3(gb), dim3(128), 0, c->stream, (const R*)L.Eb, (const R*)c->adj_cy,
                              (R*)c->Q, c->nx, c->ny, c->nz, (R)(0.5 / c->dx), (R)(0.5 / c->dz));
             TRIBO_LAUNCHED(c);
             if ((st = poisson_solve(c, c->Q, false, c->d_scale_q, true, L.psi, nullptr))) return st;
             phase_begin(c, PH_ADJOINT);
-            (void)launch_pdl(k_adj_deposit<R>, dim3(grid_for(n)), dim3(kThreads), 0, c->stream, a, L.seg[i], n,
+            (void)launch_pdl(k_adj_deposit<R>, dim3(grid_for(n)), dim3(kThreads), 0, c->stream, a, segS(i), n,
                              (const double*)L.psi, L.lam.q, reinterpret_cast<uint2*>(L.Eb),
                              (int64_t)(eb_bytes / sizeof(uint2)));
             TRIBO_LAUNCHED(c);

@@ -37,8 +37,9 @@ namespace {
 // the gather is 60 and the two divisions 18, 0.23 ms of the pipe for 1M particles.  Measured 295 us
 // (481 before the locate, the compares, the wrap and expm1 left the FP64 pipe); 80 registers, three
 // blocks a SM, hold it without spilling.  FP32: see the loop.
-template <class R>
-__global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(StepArgs<R> a, PView p, int write_cell) {
+template <class R, bool kOut = false>
+__global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(StepArgs<R> a, PView p, int write_cell,
+                                                                             PView o) {
     pdl_wait();
     extern __shared__ unsigned int sh_hist[];
     const bool use_hist = a.hist != nullptr;
@@ -53,7 +54,7 @@ __global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(Ste
     // still in L2), and the charge sums deposited last are the ones the next solve reads first
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < p.n; m += stride)
-        step_one<R>(a, p, p.n - 1 - m, write_cell, sh_hist, use_hist, err);
+        step_one<R, kOut>(a, p, p.n - 1 - m, write_cell, sh_hist, use_hist, err, kOut ? &o : nullptr);
     if (err) atomicOr(&a.acc->err, err);
     if (use_hist) {
         __syncthreads();
@@ -124,7 +125,10 @@ tribo_status step_impl(tribo_ctx* c, const PView& p, double dt, bool deposit_nex
     const int threads = p.n <= (int64_t)c->num_sms * kStepThreads ? 64 : kStepThreads;
     const int kblocks = (int)std::min<int64_t>((p.n + threads - 1) / threads,
                                                (int64_t)c->num_sms * step_min_blocks<R>() * (kStepThreads / threads));
-    (void)launch_pdl(k_step<R>, dim3(kblocks), dim3(threads), sh, c->stream, a, p, write_cell ? 1 : 0);
+    if (io.out)
+        (void)launch_pdl(k_step<R, true>, dim3(kblocks), dim3(threads), sh, c->stream, a, p, write_cell ? 1 : 0, *io.out);
+    else
+        (void)launch_pdl(k_step<R>, dim3(kblocks), dim3(threads), sh, c->stream, a, p, write_cell ? 1 : 0, PView{});
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
 }
@@ -465,8 +469,10 @@ tribo_status lattice_from_aos3(tribo_ctx* c, const void* src_dev) {
 }
 
 tribo_status particles_setup(tribo_ctx* c) {
-    TRIBO_CUDA(cudaFuncSetAttribute(k_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 1024 * 4));
-    TRIBO_CUDA(cudaFuncSetAttribute(k_step<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 1024 * 4));
+    (void)c;
+    const void* fns[] = {(const void*)k_step<float>, (const void*)k_step<double>, (const void*)k_step<float, true>,
+                         (const void*)k_step<double, true>};
+    for (const void* f : fns) TRIBO_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 1024 * 4));
     return TRIBO_OK;
 }
 

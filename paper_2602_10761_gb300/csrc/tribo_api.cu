@@ -410,7 +410,7 @@ void free_ctx(tribo_ctx* c) {
                     c->d_xf, c->d_zf, c->d_ybin, c->d_Yr, c->d_invdY, c->d_yrow, c->u_lat, c->E_lat, c->Q, c->stage, c->d_acc,
                     c->d_hist, c->d_scalar, c->alt, c->sort_counts, c->sort_key, c->sort_rank, c->sort_perm,
                     c->sort_tiles, c->adj, c->nf_members, c->nf_acc, c->pp_partner, c->d_inv_vol,
-                    c->adj_E, c->n_imp0, c->patch};
+                    c->adj_cy, c->adj_E, c->n_imp0, c->patch};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);

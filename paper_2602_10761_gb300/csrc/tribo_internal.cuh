@@ -162,7 +162,8 @@ struct tribo_ctx {
     void* d_inv_vol = nullptr;         // 1 / (dx dy_j dz) per y cell, real type
     void* adj = nullptr;               // adjoint workspace (checkpoints, segment states, adjoints)
     size_t adj_bytes = 0;
-    void* adj_E = nullptr;             // adjoint: the field of every forward step, when it fits
+    void* adj_cy = nullptr;            // adjoint: transposed gradient's y coefficients, real type
+    void* adj_E = nullptr;             // adjoint: the field and the state of every forward step, as far as they fit
     size_t adj_E_bytes = 0;
     int64_t adj_E_limit = -1;          // its budget: < 0 half of the free memory, else bytes
 
@@ -319,6 +320,7 @@ struct StepIO {               // per-call overrides of the context's buffers
     const void* acoul = nullptr; // near-field acceleration planes (x, y, z) or NULL
     void* fs = nullptr;          // momentum source planes to add this step's drag to, or NULL
     double fs_coef = 0.0;        // -1 / (rho dt nsteps): the mean over the call's steps
+    const PView* out = nullptr;  // where the new positions, velocities and charges go (NULL: in place)
 };
 tribo_status particles_step(tribo_ctx* c, const PView& p, double dt, bool deposit_next,
                             bool write_cell, const StepIO& io = StepIO());
