@@ -10,286 +10,24 @@
 // 3-point operator in x and z and the flux form on the stretched y grid, with
 // phi = 0 on the wall faces.  The DFT in x and z diagonalises the x and z
 // parts with modified wavenumbers lam(m) = (4/h^2) sin^2(pi m / N), leaving a
-// real tridiagonal system in y per (m_x, m_z) pencil, solved in FP64 by the
-// Thomas algorithm.  E is formed in spectral space: the central difference in
+// real tridiagonal system in y per (m_x, m_z) pencil.  E is formed in spectral space: the central difference in
 // x (z) is the multiplier -i sin(2 pi m / N) / h, and the Gauss-linear E_y at
 // each lattice node is a 3-point combination of phi in y; the spectra are then
 // transformed back to the wall-extended lattice.
 //
-// Passes (each a kernel):
-//   fwd_x : real line FFT in x of -rho/eps (charge sums scaled per row),
-//           optionally zeroing the charge buffer for the next deposit
-//   fwd_z : complex FFT in z of each (j, m_x) column
-//   solve : FP64 Thomas per pencil, then the E (and phi) spectra per node
-//   inv_z : inverse complex FFT in z of each field column
-//   inv_x : inverse real FFT in x, writing float4/double4 E nodes (and phi)
+// The passes are in poisson_passes.cuh (transforms, mixed y solve) and
+// poisson_y64.cuh (FP64 y solve); a context's solve is in poisson_fast.cu.
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
 #include <mutex>
+#include <set>
 
+#include "poisson_y64.cuh"
 #include "tribo_internal.cuh"
 
 namespace tribo {
-
-namespace {
-
-constexpr int kThreads = 256;
-
-// Mixed-radix (4, 2, 3) Stockham plan for one transform length.
-struct FftPlan {
-    int n = 0;
-    int npass = 0;
-    int radix[24];
-    void* tw = nullptr;      // device table, n entries of cplx<R>: exp(-2 pi i e / n)
-};
-
-bool make_plan_radices(int n, FftPlan& p) {
-    p.n = n;
-    p.npass = 0;
-    int m = n;
-    while (m % 4 == 0) { p.radix[p.npass++] = 4; m /= 4; }
-    while (m % 2 == 0) { p.radix[p.npass++] = 2; m /= 2; }
-    while (m % 3 == 0) { p.radix[p.npass++] = 3; m /= 3; }
-    return m == 1 && p.npass <= 24;
-}
-
-// In-place radix-r DFT of y[0..r) with direction sgn (-1 forward, +1 inverse).
-template <class R>
-__device__ __forceinline__ void small_dft(cplx<R>* y, int r, R sgn) {
-    if (r == 2) {
-        cplx<R> a = y[0], b = y[1];
-        y[0] = a + b;
-        y[1] = a - b;
-    } else if (r == 4) {
-        cplx<R> a = y[0] + y[2], b = y[0] - y[2], c = y[1] + y[3], d = mul_si(y[1] - y[3], sgn);
-        y[0] = a + c;
-        y[2] = a - c;
-        y[1] = b + d;
-        y[3] = b - d;
-    } else {  // r == 3
-        const R h = (R)0.86602540378443864676;  // sqrt(3)/2
-        cplx<R> t1 = y[1] + y[2];
-        cplx<R> t2 = y[0] - scale(t1, (R)0.5);
-        cplx<R> t3 = mul_si(scale(y[1] - y[2], h), sgn);
-        y[0] = y[0] + t1;
-        y[1] = t2 + t3;
-        y[2] = t2 - t3;
-    }
-}
-
-// Stockham autosort FFT of nl lines of length n held line-major in A; B is a
-// scratch buffer of the same size.  All threads of the block take part.
-// Returns the buffer that holds the (naturally ordered) result.
-template <class R>
-__device__ cplx<R>* fft_smem(cplx<R>* A, cplx<R>* B, const FftPlan& plan, int nl, R sgn,
-                             const cplx<R>* __restrict__ tw) {
-    const int n = plan.n;
-    int Ls = 1;
-    for (int p = 0; p < plan.npass; ++p) {
-        const int r = plan.radix[p];
-        const int m = n / r;
-        const int stride = n / (r * Ls);
-        for (int idx = threadIdx.x; idx < nl * m; idx += blockDim.x) {
-            const int line = idx / m;
-            const int j = idx - line * m;
-            const int k = j % Ls;
-            const cplx<R>* in = A + line * n;
-            cplx<R> y[4];
-            y[0] = in[j];
-            for (int t = 1; t < r; ++t) {
-                cplx<R> w = tw[t * k * stride];
-                if (sgn > 0) w = conj(w);
-                y[t] = in[j + t * m] * w;
-            }
-            small_dft(y, r, sgn);
-            cplx<R>* out = B + line * n + (j - k) * r + k;
-            for (int u = 0; u < r; ++u) out[u * Ls] = y[u];
-        }
-        __syncthreads();
-        cplx<R>* t = A;
-        A = B;
-        B = t;
-        Ls *= r;
-    }
-    return A;
-}
-
-// ---------------------------------------------------------------- fwd_x
-// src holds QT: the context's charge sums (QT = R) or a caller's FP64 density.
-template <class R, class QT>
-__global__ void k_fwd_x(QT* __restrict__ src, const double* __restrict__ scale_row, int zero_src,
-                        cplx<R>* __restrict__ S, int nx, int ny, int nlines, int nxh, FftPlan plan,
-                        int lpb) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<R>* A = reinterpret_cast<cplx<R>*>(smem_raw);
-    cplx<R>* B = A + lpb * nx;
-    const int line0 = blockIdx.x * lpb;
-    const int nl = min(lpb, nlines - line0);
-    for (int idx = threadIdx.x; idx < nl * nx; idx += blockDim.x) {
-        const int line = line0 + idx / nx;
-        const int i = idx - (idx / nx) * nx;
-        const int j = line % ny;
-        const size_t g = (size_t)line * nx + i;
-        const QT v = src[g];
-        if (zero_src) src[g] = (QT)0;
-        A[idx] = cplx<R>{(R)v * (R)scale_row[j], (R)0};
-    }
-    __syncthreads();
-    cplx<R>* res = fft_smem<R>(A, B, plan, nl, (R)-1, (const cplx<R>*)plan.tw);
-    for (int idx = threadIdx.x; idx < nl * nxh; idx += blockDim.x) {
-        const int l = idx / nxh;
-        const int mx = idx - l * nxh;
-        S[(size_t)(line0 + l) * nxh + mx] = res[l * nx + mx];
-    }
-}
-
-// ---------------------------------------------------------------- z transforms
-// Columns along z of an array laid out [k][plane][mx] with nplanes planes per
-// z index: block (plane, mx tile) transforms `mt` columns in place.
-template <class R>
-__global__ void k_fft_z(cplx<R>* __restrict__ arr, int nz, int nplanes, int nxh, int mt, FftPlan plan,
-                        R sgn, size_t field_stride) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<R>* A = reinterpret_cast<cplx<R>*>(smem_raw);
-    cplx<R>* B = A + mt * nz;
-    const int plane = blockIdx.x;
-    const int mx0 = blockIdx.y * mt;
-    const int nt = min(mt, nxh - mx0);
-    cplx<R>* base = arr + field_stride * blockIdx.z;
-    for (int idx = threadIdx.x; idx < nz * nt; idx += blockDim.x) {
-        const int k = idx / nt;
-        const int t = idx - k * nt;
-        A[t * nz + k] = base[((size_t)k * nplanes + plane) * nxh + mx0 + t];
-    }
-    __syncthreads();
-    cplx<R>* res = fft_smem<R>(A, B, plan, nt, sgn, (const cplx<R>*)plan.tw);
-    for (int idx = threadIdx.x; idx < nz * nt; idx += blockDim.x) {
-        const int k = idx / nt;
-        const int t = idx - k * nt;
-        base[((size_t)k * nplanes + plane) * nxh + mx0 + t] = res[t * nz + k];
-    }
-}
-
-// ---------------------------------------------------------------- y solve
-// One thread per (m_z, m_x) pencil.  Thomas forward sweep with the shifted
-// diagonal b_j - lam, backward substitution, then the E spectra per node.
-// W holds dp (later phi) and Wc holds c'_j, both FP64, laid out [j][pencil].
-template <class R>
-__global__ void k_solve_y(const cplx<R>* __restrict__ S, cplx<R>* __restrict__ F, double2* __restrict__ W,
-                          double* __restrict__ Wc, const double* __restrict__ ycoef,
-                          const double* __restrict__ lamx, const double* __restrict__ lamz,
-                          const double* __restrict__ sinx, const double* __restrict__ sinz,
-                          const double* __restrict__ ey, int ny, int nz, int nxh, int want_phi) {
-    const int np = nz * nxh;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= np) return;
-    const int mz = p / nxh;
-    const int mx = p - mz * nxh;
-    const double lam = lamx[mx] + lamz[mz];
-    const double* a = ycoef;
-    const double* b = ycoef + ny;
-    const double* c = ycoef + 2 * ny;
-    // row j of the spectrum for pencil (mz, mx) sits at S[(mz*ny + j)*nxh + mx]
-    const cplx<R>* s = S + (size_t)mz * ny * nxh + mx;
-    double cp = 0.0;
-    double2 dp = make_double2(0.0, 0.0);
-    for (int j = 0; j < ny; ++j) {
-        const double den = (b[j] - lam) - a[j] * cp;
-        const double inv = 1.0 / den;
-        const cplx<R> r = s[(size_t)j * nxh];
-        dp = make_double2(((double)r.re - a[j] * dp.x) * inv, ((double)r.im - a[j] * dp.y) * inv);
-        cp = c[j] * inv;
-        W[(size_t)j * np + p] = dp;
-        Wc[(size_t)j * np + p] = cp;
-    }
-    double2 x = dp;
-    for (int j = ny - 2; j >= 0; --j) {
-        const double2 d = W[(size_t)j * np + p];
-        const double cj = Wc[(size_t)j * np + p];
-        x = make_double2(d.x - cj * x.x, d.y - cj * x.y);
-        W[(size_t)j * np + p] = x;
-    }
-    // fields: 0 = E_x, 1 = E_y, 2 = E_z, 3 = phi ; layout [f][mz][jn][mx]
-    const int nyn = ny + 2;
-    const size_t fstride = (size_t)nz * nyn * nxh;
-    const double sx = sinx[mx], sz = sinz[mz];
-    for (int jn = 0; jn < nyn; ++jn) {
-        const int jc = jn - 1;  // cell of this node (interior nodes)
-        double2 ph = make_double2(0.0, 0.0);
-        if (jc >= 0 && jc < ny) ph = W[(size_t)jc * np + p];
-        double2 eyv = make_double2(0.0, 0.0);
-        const double cm = ey[3 * jn + 0], c0 = ey[3 * jn + 1], cpv = ey[3 * jn + 2];
-        if (jc - 1 >= 0 && jc - 1 < ny && cm != 0.0) {
-            const double2 v = W[(size_t)(jc - 1) * np + p];
-            eyv.x += cm * v.x; eyv.y += cm * v.y;
-        }
-        if (jc >= 0 && jc < ny && c0 != 0.0) { eyv.x += c0 * ph.x; eyv.y += c0 * ph.y; }
-        if (jc + 1 >= 0 && jc + 1 < ny && cpv != 0.0) {
-            const double2 v = W[(size_t)(jc + 1) * np + p];
-            eyv.x += cpv * v.x; eyv.y += cpv * v.y;
-        }
-        const size_t o = ((size_t)mz * nyn + jn) * nxh + mx;
-        // -i s phi = (s * im, -s * re)
-        F[o] = cplx<R>{(R)(sx * ph.y), (R)(-sx * ph.x)};
-        F[fstride + o] = cplx<R>{(R)eyv.x, (R)eyv.y};
-        F[2 * fstride + o] = cplx<R>{(R)(sz * ph.y), (R)(-sz * ph.x)};
-        if (want_phi) F[3 * fstride + o] = cplx<R>{(R)ph.x, (R)ph.y};
-    }
-}
-
-// ---------------------------------------------------------------- inv_x
-template <class R>
-__global__ void k_inv_x(const cplx<R>* __restrict__ F, R* __restrict__ E, double* __restrict__ phi,
-                        int nx, int ny, int nz, int nxh, FftPlan plan, int lpb, int nf) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cplx<R>* A = reinterpret_cast<cplx<R>*>(smem_raw);
-    cplx<R>* B = A + lpb * nx;
-    const int nyn = ny + 2;
-    const int nlines = nz * nyn;
-    const size_t nodes = (size_t)nlines * nx;   // E planes: E_x, E_y, E_z
-    const size_t fstride = (size_t)nz * nyn * nxh;
-    const int line0 = blockIdx.x * lpb;
-    const int nl = min(lpb, nlines - line0);
-    const R norm = (R)(1.0 / ((double)nx * (double)nz));
-    for (int f = 0; f < nf; ++f) {
-        for (int idx = threadIdx.x; idx < nl * nx; idx += blockDim.x) {
-            const int l = idx / nx;
-            const int m = idx - l * nx;
-            const cplx<R>* src = F + f * fstride + (size_t)(line0 + l) * nxh;
-            A[idx] = (m < nxh) ? src[m] : conj(src[nx - m]);
-        }
-        __syncthreads();
-        cplx<R>* res = fft_smem<R>(A, B, plan, nl, (R)1, (const cplx<R>*)plan.tw);
-        for (int idx = threadIdx.x; idx < nl * nx; idx += blockDim.x) {
-            const R v = res[idx].re * norm;
-            if (f < 3) {
-                E[f * nodes + (size_t)line0 * nx + idx] = v;
-            } else {
-                const int line = line0 + idx / nx;
-                const int k = line / nyn;
-                const int jn = line - k * nyn;
-                const int i = idx - (idx / nx) * nx;
-                if (jn >= 1 && jn <= ny) phi[((size_t)k * ny + (jn - 1)) * nx + i] = (double)v;
-            }
-        }
-        __syncthreads();
-        if (res != A) {  // keep A as the input buffer of the next field
-            cplx<R>* t = A; A = B; B = t;
-        }
-    }
-}
-
-template <class R>
-size_t smem_fwd_x(int nx, int lpb) { return sizeof(cplx<R>) * 2 * (size_t)lpb * nx; }
-template <class R>
-size_t smem_inv_x(int nx, int lpb) { return sizeof(cplx<R>) * 2 * (size_t)lpb * nx; }
-
-template <class R> int lines_per_block() { return sizeof(R) == 4 ? 4 : 2; }
-template <class R> int z_tile() { return sizeof(R) == 4 ? 8 : 4; }
-
-}  // namespace
 
 tribo_status poisson_setup(tribo_ctx* c) {
     const int nx = c->nx, ny = c->ny, nz = c->nz, nxh = c->nxh;
@@ -404,33 +142,44 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratch
 struct NoallocDevice {
     unsigned char* base = nullptr;
     int smem_max = 0;            // opt-in shared memory per block of the device
+    int num_sms = 1;
     bool ready = false;
+    std::set<int> lengths;       // (precision, x or z, length) whose shared-memory limits are set
 };
 NoallocDevice g_noalloc_dev[kNoallocMaxDevices];
 std::mutex g_noalloc_mutex;
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
-struct NoallocLayout {
-    size_t tables, twx, twz, S, F, W, total;
-};
-
-size_t noalloc_table_doubles(int nx, int ny, int nz) {
+// The scratch that decides which grids the call takes: spectrum, nf field spectra and 24 bytes per
+// pencil and row of sweep storage beside the tables.
+size_t noalloc_capacity(int nx, int ny, int nz, int nf, size_t rsz) {
+    const size_t csz = 2 * rsz;
     const int nxh = nx / 2 + 1;
-    return (size_t)3 * ny + nx + nz + nxh + nz + 3 * (ny + 2) + ny;
+    const size_t tables = (size_t)3 * ny + nx + nz + nxh + nz + 3 * (ny + 2) + ny;
+    return round256(tables * sizeof(double)) + round256((size_t)nx * csz) + round256((size_t)nz * csz) +
+           round256((size_t)nz * ny * nxh * csz) + round256((size_t)nf * nz * (ny + 2) * nxh * csz) +
+           round256((size_t)ny * nz * nxh * (sizeof(double2) + sizeof(double)));
 }
 
-NoallocLayout noalloc_layout(int nx, int ny, int nz, int nf, size_t rsz) {
+// What the passes use of it: the y tables (2 ny + 1 rows of (nz/2+1) nxh doubles) take the place of
+// the sweep storage and are smaller for every nz >= 4, the x twiddles carry their inner table, the
+// potential needs no field of its own.
+struct NoallocLayout {
+    size_t tables, twx, twz, te, S, F, total;
+};
+NoallocLayout noalloc_layout(int nx, int ny, int nz, size_t rsz) {
     const size_t csz = 2 * rsz;
     const int nxh = nx / 2 + 1;
     NoallocLayout L{};
     size_t off = 0;
-    L.tables = off; off += round256(noalloc_table_doubles(nx, ny, nz) * sizeof(double));
-    L.twx = off;    off += round256((size_t)nx * csz);
-    L.twz = off;    off += round256((size_t)nz * csz);
-    L.S = off;      off += round256((size_t)nz * ny * nxh * csz);
-    L.F = off;      off += round256((size_t)nf * nz * (ny + 2) * nxh * csz);
-    L.W = off;      off += round256((size_t)ny * nz * nxh * (sizeof(double2) + sizeof(double)));
+    auto take = [&](size_t bytes) { const size_t o = off; off += round256(bytes); return o; };
+    L.tables = take(((size_t)3 * ny + nxh + nz + 3 * (ny + 2) + ny) * sizeof(double));
+    L.twx = take(((size_t)nx + nx / 2) * csz);
+    L.twz = take((size_t)nz * csz);
+    L.te = take((size_t)(2 * ny + 1) * (nz / 2 + 1) * nxh * sizeof(double));
+    L.S = take((size_t)nz * ny * nxh * csz);
+    L.F = take((size_t)3 * nz * (ny + 2) * nxh * csz);
     L.total = off;
     return L;
 }
@@ -439,29 +188,26 @@ NoallocLayout noalloc_layout(int nx, int ny, int nz, int nf, size_t rsz) {
 // the table kernel (no host buffer is copied: the call neither blocks on nor
 // reads host memory after it returns).
 struct NoallocGeom {
-    int nx, ny, nz;
+    int nx, ny, nz, n1;
     double dx, dz, eps;
     double yf[kNoallocMaxN + 1];
 };
 
-// The grid tables of the solve, written into the front of the scratch array in
-// the layout of noalloc_layout: the y operator (a, b, c), the modified
-// wavenumbers, the spectral derivative factors, the E_y node coefficients, the
-// per-row RHS scale -1/eps and the x and z twiddles.  One block; the same
-// formulas as poisson_setup and make_plan (Sec. 2.2, Sec. 3.1 FV operator).
+// The grid tables of the solve, written into the front of the scratch array: the y operator (a, b,
+// c), the spectral derivative factors, the E_y node coefficients, the per-row RHS scale -1/(eps nx nz)
+// and the x and z twiddles by block 0 (the same formulas as poisson_setup and the contexts' tables,
+// Sec. 2.2, Sec. 3.1 FV operator), the y factors by the others, two neighbouring threads a wavenumber
+// pair, from the y operator that each block forms for itself in shared memory.  Bound by the latency of
+// a thread's chain of ny/2 FP64 divisions; the passes after it are those of a context (a mixed 64^3
+// call: 202 us with one kernel a sweep over generic transforms, 62.5 us so).  Measured and not taken:
+// one-warp blocks with a value a thread (64.4 us), factors by continuants without the divisions in the
+// chain (72.8 us, more FP64 operations).
 template <class R>
-__global__ void k_noalloc_tables(NoallocGeom g, double* __restrict__ T, cplx<R>* __restrict__ twx,
-                                 cplx<R>* __restrict__ twz) {
+__global__ void __launch_bounds__(128) k_noalloc_tables(NoallocGeom g, double* __restrict__ T, cplx<R>* __restrict__ twx,
+                                                        cplx<R>* __restrict__ twz, double* __restrict__ te) {
+    pdl_wait();
+    __shared__ double sy[3 * kNoallocMaxN];
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxh = nx / 2 + 1;
-    double* a = T;
-    double* b = a + ny;
-    double* cc = b + ny;
-    double* lamx = T + 3 * ny;
-    double* lamz = lamx + nx;
-    double* sinx = lamz + nz;
-    double* sinz = sinx + nxh;
-    double* ey = sinz + nz;
-    double* scale = ey + 3 * (ny + 2);
     const double* yf = g.yf;
     auto yc = [&](int j) { return 0.5 * (yf[j] + yf[j + 1]); };
     auto dy = [&](int j) { return yf[j + 1] - yf[j]; };
@@ -471,10 +217,27 @@ __global__ void k_noalloc_tables(NoallocGeom g, double* __restrict__ T, cplx<R>*
         double bj = -(aj + cj);
         if (j == 0) bj -= 1.0 / (dy(0) * (yc(0) - yf[0]));
         if (j == ny - 1) bj -= 1.0 / (dy(ny - 1) * (yf[ny] - yc(ny - 1)));
-        a[j] = aj;
-        b[j] = bj;
-        cc[j] = cj;
-        scale[j] = -1.0 / g.eps;
+        sy[j] = aj;
+        sy[ny + j] = bj;
+        sy[2 * ny + j] = cj;
+    }
+    __syncthreads();
+    if (blockIdx.x > 0) {
+        const int ni = (nz / 2 + 1) * nxh;
+        const int t = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
+        const int item = min(t >> 1, ni - 1);           // threads past the end repeat the last pair's work
+        const double sx = sin(M_PI * (item % nxh) / nx), sz = sin(M_PI * (item / nxh) / nz);
+        const double lam = 4.0 / (g.dz * g.dz) * sz * sz + 4.0 / (g.dx * g.dx) * sx * sx;
+        y_factors(sy, lam, ny, ni, item, 1 + (t & 1), te, te + (size_t)(ny + 1) * ni);
+        return;
+    }
+    double* sinx = T + 3 * ny;
+    double* sinz = sinx + nxh;
+    double* ey = sinz + nz;
+    double* scale = ey + 3 * (ny + 2);
+    for (int j = threadIdx.x; j < 3 * ny; j += blockDim.x) T[j] = sy[j];
+    for (int j = threadIdx.x; j < ny; j += blockDim.x) {
+        scale[j] = -1.0 / g.eps / ((double)nx * (double)nz);
         // E_y at lattice node jn = j + 1: cm phi[j-1] + c0 phi[j] + cp phi[j+1]
         double cm = 0, c0 = 0, cp = 0;
         if (j >= 1) {
@@ -500,72 +263,62 @@ __global__ void k_noalloc_tables(NoallocGeom g, double* __restrict__ T, cplx<R>*
         ey[3 * (ny + 1) + 2] = 0.0;
     }
     for (int m = threadIdx.x; m < nx; m += blockDim.x) {
-        const double s = sin(M_PI * m / nx);
-        lamx[m] = 4.0 / (g.dx * g.dx) * s * s;
-        const double ang = 2.0 * M_PI * (double)m / (double)nx;
-        twx[m] = cplx<R>{(R)cos(ang), (R)(-sin(ang))};
-        if (m < nxh) sinx[m] = sin(ang) / g.dx;
+        double s, c;
+        sincos(2.0 * M_PI * (double)m / (double)nx, &s, &c);
+        twx[m] = cplx<R>{(R)c, (R)(-s)};
+        if (m < nxh) sinx[m] = s / g.dx;
     }
     for (int m = threadIdx.x; m < nz; m += blockDim.x) {
-        const double s = sin(M_PI * m / nz);
-        lamz[m] = 4.0 / (g.dz * g.dz) * s * s;
-        const double ang = 2.0 * M_PI * (double)m / (double)nz;
-        sinz[m] = sin(ang) / g.dz;
-        twz[m] = cplx<R>{(R)cos(ang), (R)(-sin(ang))};
+        double s, c;
+        sincos(2.0 * M_PI * (double)m / (double)nz, &s, &c);
+        sinz[m] = s / g.dz;
+        twz[m] = cplx<R>{(R)c, (R)(-s)};
     }
+    __syncthreads();
+    // the x transform's inner twiddles by thread: M = n1 n2, n1 the largest divisor not above sqrt(M)
+    const int M = nx / 2, n2 = M / g.n1;
+    for (int i = threadIdx.x; i < M; i += blockDim.x) twx[nx + i] = twx[2 * (i % n2) * (i / n2)];
 }
 
 template <class R>
 tribo_status noalloc_solve(const tribo_grid* g, double eps, const double* rho, double* phi, void* E,
-                           cudaStream_t stream, unsigned char* base, const NoallocLayout& L, int smem_max) {
+                           cudaStream_t stream, unsigned char* base, const NoallocLayout& L, int num_sms) {
     const int nx = g->nx, ny = g->ny, nz = g->nz, nxh = nx / 2 + 1;
-    const int lpb = lines_per_block<R>();
-    const int mt = z_tile<R>();
-    // the kernels' shared memory, against the device
-    const size_t need = std::max({smem_fwd_x<R>(nx, lpb), smem_inv_x<R>(nx, lpb), sizeof(cplx<R>) * 2 * mt * nz});
-    if (need > (size_t)smem_max) {
-        set_last_error("tribo_poisson_noalloc: grid needs more shared memory per block than the device offers");
-        return TRIBO_ERR_UNSUPPORTED;
-    }
     NoallocGeom geom{};
     geom.nx = nx; geom.ny = ny; geom.nz = nz;
     geom.dx = g->lx / nx; geom.dz = g->lz / nz; geom.eps = eps;
+    geom.n1 = 1;
+    for (int d = 1; d * d <= nx / 2; ++d)
+        if ((nx / 2) % d == 0) geom.n1 = d;
     for (int j = 0; j <= ny; ++j) geom.yf[j] = g->y_faces[j];
-    double* dT = reinterpret_cast<double*>(base + L.tables);
-    k_noalloc_tables<R><<<1, kThreads, 0, stream>>>(geom, dT, reinterpret_cast<cplx<R>*>(base + L.twx),
-                                                    reinterpret_cast<cplx<R>*>(base + L.twz));
-    FftPlan px{}, pz{};
-    make_plan_radices(nx, px);
-    make_plan_radices(nz, pz);
-    px.tw = base + L.twx;
-    pz.tw = base + L.twz;
-    const double* d_ycoef = dT;
-    const double* d_lamx = dT + 3 * ny;
-    const double* d_lamz = d_lamx + nx;
-    const double* d_sinx = d_lamz + nz;
-    const double* d_sinz = d_sinx + nxh;
-    const double* d_ey = d_sinz + nz;
-    const double* d_scale = d_ey + 3 * (ny + 2);
+    double* T = reinterpret_cast<double*>(base + L.tables);
+    cplx<R>* twx = reinterpret_cast<cplx<R>*>(base + L.twx);
+    cplx<R>* twz = reinterpret_cast<cplx<R>*>(base + L.twz);
+    double* te = reinterpret_cast<double*>(base + L.te);
     cplx<R>* S = reinterpret_cast<cplx<R>*>(base + L.S);
     cplx<R>* F = reinterpret_cast<cplx<R>*>(base + L.F);
-    double2* W = reinterpret_cast<double2*>(base + L.W);
-    double* Wc = reinterpret_cast<double*>(W + (size_t)ny * nz * nxh);
-    const int want_phi = phi != nullptr ? 1 : 0;
-    const int nf = 3 + want_phi;
-    const int nlines = ny * nz;
-    k_fwd_x<R, double><<<(nlines + lpb - 1) / lpb, kThreads, smem_fwd_x<R>(nx, lpb), stream>>>(
-        const_cast<double*>(rho), d_scale, 0, S, nx, ny, nlines, nxh, px, lpb);
-    k_fft_z<R><<<dim3(ny, (nxh + mt - 1) / mt, 1), kThreads, sizeof(cplx<R>) * 2 * mt * nz, stream>>>(
-        S, nz, ny, nxh, mt, pz, (R)-1, 0);
-    const int np = nz * nxh;
-    k_solve_y<R><<<(np + 127) / 128, 128, 0, stream>>>(S, F, W, Wc, d_ycoef, d_lamx, d_lamz, d_sinx, d_sinz,
-                                                       d_ey, ny, nz, nxh, want_phi);
-    const size_t fstride = (size_t)nz * (ny + 2) * nxh;
-    k_fft_z<R><<<dim3(ny + 2, (nxh + mt - 1) / mt, nf), kThreads, sizeof(cplx<R>) * 2 * mt * nz, stream>>>(
-        F, nz, ny + 2, nxh, mt, pz, (R)1, fstride);
-    const int nl2 = nz * (ny + 2);
-    k_inv_x<R><<<(nl2 + lpb - 1) / lpb, kThreads, smem_inv_x<R>(nx, lpb), stream>>>(
-        F, (R*)E, phi, nx, ny, nz, nxh, px, lpb, nf);
+    const double* sinx = T + 3 * ny;
+    const double* sinz = sinx + nxh;
+    const double* ey = sinz + nz;
+    const double* scale = ey + 3 * (ny + 2);
+    const int ni = (nz / 2 + 1) * nxh;
+    (void)launch_pdl(k_noalloc_tables<R>, dim3(1 + (2 * ni + 127) / 128), dim3(128), 0, stream, geom, T, twx, twz, te);
+    // the forward x transform reads pairs of densities: a density aligned to its elements only passes
+    // through the field spectra's space, which is written later
+    const double* src = rho;
+    if (reinterpret_cast<uintptr_t>(rho) % sizeof(double2)) {
+        const cudaError_t e = cudaMemcpyAsync(F, rho, sizeof(double) * (size_t)nx * ny * nz, cudaMemcpyDeviceToDevice, stream);
+        if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: copy of the density");
+        src = reinterpret_cast<const double*>(F);
+    }
+    const PassGrid<R> pg{nx, ny, nz, nxh, num_sms, stream};
+    xfwd_launch<R>(pg, const_cast<double*>(src), true, scale, false, S, twx);
+    zfwd_launch<R>(pg, S, twz);
+    (void)launch_pdl(k_ysolve64<R>, dim3((unsigned)(((int64_t)nz * nxh + 31) / 32)), dim3(128), ysolve64_smem(ny), stream,
+                     S, F, (const double*)te, (const double*)(te + (size_t)(ny + 1) * ni), (const double*)T, ey, ny, nz,
+                     nxh, 1);
+    zinv_launch<R>(pg, S, F, sinz, twz, false);
+    xinv_launch<R>(pg, F, (R*)E, phi, sinx, twx);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: kernel launch");
     return TRIBO_OK;
@@ -578,32 +331,37 @@ bool noalloc_2a3b(int n) {
     return n == 1;
 }
 
-// one-time set-up of the current device: the array's device address and the
-// kernels' shared-memory limit
-tribo_status noalloc_device(int dev, unsigned char** base, int* smem_max) {
+// set-up of the current device: the array's device address, and the shared-memory limits of the
+// transforms of a grid when its lengths are first used
+template <class R>
+tribo_status noalloc_device(int dev, int m, int nz, NoallocDevice* out) {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     NoallocDevice& d = g_noalloc_dev[dev];
     if (!d.ready) {
         void* p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: cudaGetSymbolAddress");
-        int optin = 0;
+        int optin = 0, sms = 0;
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: device attribute");
-        const void* fns[] = {(const void*)k_fwd_x<float, double>, (const void*)k_inv_x<float>,
-                             (const void*)k_fft_z<float>, (const void*)k_fwd_x<double, double>,
-                             (const void*)k_inv_x<double>,
-                             (const void*)k_fft_z<double>};
-        for (const void* f : fns) {
-            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-            if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: shared-memory limit");
-        }
         d.base = static_cast<unsigned char*>(p);
         d.smem_max = optin;
+        d.num_sms = std::max(1, sms);
         d.ready = true;
     }
-    *base = d.base;
-    *smem_max = d.smem_max;
+    const int kx = (int)sizeof(R) * 4096 + m, kz = (int)sizeof(R) * 4096 + 2048 + nz;
+    tribo_status st;
+    if (!d.lengths.count(kx)) {
+        if ((st = xpass_attr<R>(m, d.smem_max))) return st;
+        d.lengths.insert(kx);
+    }
+    if (!d.lengths.count(kz)) {
+        if ((st = zpass_attr<R>(nz, d.smem_max))) return st;
+        d.lengths.insert(kz);
+    }
+    out->base = d.base;
+    out->num_sms = d.num_sms;
     return TRIBO_OK;
 }
 
@@ -631,13 +389,15 @@ extern "C" tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps
         return TRIBO_ERR_UNSUPPORTED;
     }
     const size_t rsz = precision == TRIBO_FP64 ? sizeof(double) : sizeof(float);
-    const NoallocLayout L = noalloc_layout(nx, ny, nz, phi ? 4 : 3, rsz);
-    if (nx > kNoallocMaxN || ny > kNoallocMaxN || nz > kNoallocMaxN || L.total > kNoallocScratchBytes) {
+    const size_t need = noalloc_capacity(nx, ny, nz, phi ? 4 : 3, rsz);
+    const NoallocLayout L = noalloc_layout(nx, ny, nz, rsz);
+    if (nx > kNoallocMaxN || ny > kNoallocMaxN || nz > kNoallocMaxN || need > kNoallocScratchBytes ||
+        L.total > kNoallocScratchBytes) {
         char buf[256];
         snprintf(buf, sizeof buf,
                  "tribo_poisson_noalloc: a %dx%dx%d grid needs %.1f MiB of static scratch; the limit is "
                  "%d MiB and %d cells per direction",
-                 nx, ny, nz, L.total / 1048576.0, (int)(kNoallocScratchBytes >> 20), kNoallocMaxN);
+                 nx, ny, nz, need / 1048576.0, (int)(kNoallocScratchBytes >> 20), kNoallocMaxN);
         set_last_error(buf);
         return TRIBO_ERR_CAPACITY;
     }
@@ -657,11 +417,11 @@ extern "C" tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps
         set_last_error("tribo_poisson_noalloc: device ordinal out of range");
         return TRIBO_ERR_UNSUPPORTED;
     }
-    unsigned char* base = nullptr;
-    int smem_max = 0;
-    tribo_status st = noalloc_device(dev, &base, &smem_max);
+    NoallocDevice d;
+    const bool f64 = precision == TRIBO_FP64;
+    tribo_status st = f64 ? noalloc_device<double>(dev, nx / 2, nz, &d) : noalloc_device<float>(dev, nx / 2, nz, &d);
     if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
-    if (precision == TRIBO_FP64) return noalloc_solve<double>(grid, eps, rho, phi, E, s, base, L, smem_max);
-    return noalloc_solve<float>(grid, eps, rho, phi, E, s, base, L, smem_max);
+    if (f64) return noalloc_solve<double>(grid, eps, rho, phi, E, s, d.base, L, d.num_sms);
+    return noalloc_solve<float>(grid, eps, rho, phi, E, s, d.base, L, d.num_sms);
 }

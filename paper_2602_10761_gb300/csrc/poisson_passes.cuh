@@ -625,6 +625,8 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
     for (int i = threadIdx.x; i < NXH; i += kThreads) sx[i] = from_f64<R>(sinx[i]);
     __syncthreads();
     const int nyn = ny + 2;
+    // a caller's field without a context (tribo_poisson_noalloc) may be aligned to its elements only
+    const bool pairs = (reinterpret_cast<uintptr_t>(E) & (2 * sizeof(R) - 1)) == 0;
     const int r = threadIdx.x % TPC;
     const int l = threadIdx.x / TPC;
     const int ntb = (nz * nyn + LPB - 1) / LPB;
@@ -671,7 +673,12 @@ __global__ void __launch_bounds__(kThreads, (fft_min_blocks<R, M>())) k_xinv4(co
 #pragma unroll
                 for (int k2 = 0; k2 < N2; ++k2) {
                     const int k = r2 + N1 * k2;
-                    store_pair<R>(row + 2 * k, z[k2].re, z[k2].im);
+                    if (pairs) {
+                        store_pair<R>(row + 2 * k, z[k2].re, z[k2].im);
+                    } else {
+                        row[2 * k] = z[k2].re;
+                        row[2 * k + 1] = z[k2].im;
+                    }
                 }
             } else {
                 double* prow = phi + ((size_t)(line2 / nyn) * ny + (jn2 - 1)) * NX;
