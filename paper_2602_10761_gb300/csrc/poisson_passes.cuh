@@ -85,6 +85,12 @@ __device__ __forceinline__ cplx<R> split_inv_dx(cplx<R> xa, cplx<R> xb, cplx<R> 
 template <class R, int M>
 constexpr int xfwd_min_blocks() { return sizeof(R) == 4 && M <= 192 && fft::FourStep<M, kThreads>::N2 <= 16 ? 6 : 1; }
 
+// whether v is not +-0: on the bits, as a comparison of doubles would go to the FP64 pipe
+__device__ __forceinline__ bool is_nonzero(float v) { return v != 0.0f; }
+__device__ __forceinline__ bool is_nonzero(double v) {
+    return (((unsigned)__double2hiint(v) << 1) | (unsigned)__double2loint(v)) != 0u;
+}
+
 template <class R, int M, class QT, bool kTab = false>
 __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT* __restrict__ src, const double* __restrict__ scale_row,
                                                     int zero_src, cplx<R>* __restrict__ S, int ny, int nlines,
@@ -120,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
 #pragma unroll
         for (int n1 = 0; n1 < N1; ++n1) {
             const V2 v = row[N2 * n1 + r];
-            nz_mask |= (v.x != (QT)0 || v.y != (QT)0) ? 1u << n1 : 0u;
+            nz_mask |= is_nonzero(v.x) | is_nonzero(v.y) ? 1u << n1 : 0u;
             y[n1] = cplx<R>{from_f64<R>(v.x) * s, from_f64<R>(v.y) * s};
         }
         if (zero_src) {
