@@ -94,7 +94,8 @@ typedef struct {
  * dq_t: 1 to include the pre-charge transfer dq_t = -(A_iw / (pi d^2)) q
  *       (Eq. precharge-surface read as contact-area fraction), 0 to omit it.
  * electrostatics: 1 to deposit, solve and apply q E / m each step, 0 for none.
- * sort_every: re-sort particles by cell every this many steps (0 = never);
+ * sort_every: re-sort particles in space every this many steps (0 = never), by
+ *       the lattice nodes they read the fields from;
  *       sorting permutes all particle arrays, including id.
  * coulomb: 1 to add the near field of the hybrid electrostatics (Sec. 2.2):
  *       Coulomb's law between particles that share a cell, on top of the mesh
