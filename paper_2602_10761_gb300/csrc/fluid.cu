@@ -21,9 +21,9 @@
 namespace tribo {
 namespace {
 
-constexpr int kModeChunk = 256;   // modes staged in shared memory per pass
+constexpr int kModeChunk = 64;    // modes staged in shared memory per pass
 constexpr int kEvalThreads = 64;
-constexpr int kRows = 8;          // z rows per block: the x factor and amplitudes serve all of them (2: 264 us, 4: 173, 8: 139, 12: 148, 16: 154 at 128^3)
+constexpr int kRows = 8;          // z rows per block: the x factor and amplitudes serve all of them
 
 template <class R>
 __global__ void k_mode_phase(int rows, int nm, const double* __restrict__ mf, const double* __restrict__ Y,
@@ -50,19 +50,40 @@ __device__ __forceinline__ int mod_small(int v, int n, float inv_n) {
     return r;
 }
 
+// a mode's values of the block's rows, read in 16-byte loads
+template <class R>
+struct alignas(16) RowSet { cplx<R> g[kRows]; };
+
+// Place of exp(i pi l / nx) in shared memory: one value of padding after 16, so that the lanes'
+// values, 2 nxi apart, spread over the banks.
+__device__ __forceinline__ int xpad(int l) { return l + (l >> 4); }
+template <class R>
+size_t eval_smem(int nx) { return sizeof(cplx<R>) * (size_t)(2 * nx + (2 * nx) / 16 + 1); }
+
+// Bound by FP32 issue: 80 operations a mode and thread, 70 us of the pipe at 128^3 with 256 modes.
+// Read from global memory the x factors, nxi values apart, kept the L1 data pipe as busy as the
+// arithmetic by their bank conflicts; they come from a padded copy in shared memory, found by a
+// multiplication instead of a division by float, with the rows' values side by side and four modes in
+// flight: 123 -> 108 us, the same sums in the same order.  (128 or 256 modes staged: 110-112; two in
+// flight: 115; the factors mode by mode in a table of their own: 111 alone, but 135 within a step.)
 template <class R>
 __global__ void __launch_bounds__(kEvalThreads)
 k_mode_eval(int nx, int ny2, int nz, int nm, const int2* __restrict__ ma, const double* __restrict__ mf,
             const cplx<R>* __restrict__ mc, const cplx<R>* __restrict__ tabx, const cplx<R>* __restrict__ tabz,
             const double* __restrict__ ubar, R* __restrict__ out) {
     pdl_wait();
-    __shared__ cplx<R> G[kRows][kModeChunk];      // c_m(jn) Z_m(k) per row of the block
+    __shared__ RowSet<R> G[kModeChunk];           // c_m(jn) Z_m(k) per row of the block
     __shared__ vec4<R> A[kModeChunk];             // amplitude vector
     __shared__ int AX[kModeChunk];                // nxi mod 2 nx
     const int k0 = blockIdx.x * kRows, jn = blockIdx.y;
     const int nrow = min(kRows, nz - k0);
     const int n2x = 2 * nx, n2z = 2 * nz;
-    const float inv2x = 1.0f / (float)n2x, inv2z = 1.0f / (float)n2z;
+    const float inv2z = 1.0f / (float)n2z;
+    // v mod 2 nx = v - 2 nx (v magic >> 32) for v < 2 nx^2: exact as v (magic 2 nx - 2^32) <= v 2 nx < 2^32
+    const unsigned magic = 0xffffffffu / (unsigned)n2x + 1u;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cplx<R>* sx = reinterpret_cast<cplx<R>*>(smem_raw);
+    for (int l = threadIdx.x; l < n2x; l += kEvalThreads) sx[xpad(l)] = tabx[l];
     const int npair = nx / 2;
     const size_t plane = (size_t)nz * ny2 * nx;
     const R ub = from_f64<R>(ubar[jn]);
@@ -83,21 +104,23 @@ k_mode_eval(int nx, int ny2, int nz, int nm, const int2* __restrict__ ma, const 
                 const cplx<R> cm = mc[(size_t)jn * nm + m];
 #pragma unroll
                 for (int r = 0; r < kRows; ++r)
-                    G[r][e] = r < nrow ? cm * tabz[mod_small(am.y * (2 * (k0 + r) + 1), n2z, inv2z)]
-                                       : cplx<R>{0, 0};
+                    G[e].g[r] = r < nrow ? cm * tabz[mod_small(am.y * (2 * (k0 + r) + 1), n2z, inv2z)]
+                                         : cplx<R>{0, 0};
                 A[e] = vec4<R>{from_f64<R>(mf[6 * m + 3]), from_f64<R>(mf[6 * m + 4]), from_f64<R>(mf[6 * m + 5]),
                                (R)0};
                 AX[e] = am.x;
             }
             __syncthreads();
             if (i < npair) {
-#pragma unroll 2
+#pragma unroll 4
                 for (int e = 0; e < cnt; ++e) {
-                    const cplx<R> X = tabx[mod_small(AX[e] * ii, n2x, inv2x)];
+                    const unsigned v = (unsigned)(AX[e] * ii);
+                    const cplx<R> X = sx[xpad((int)(v - __umulhi(v, magic) * (unsigned)n2x))];
                     const vec4<R> av = A[e];
+                    const RowSet<R> gs = G[e];
 #pragma unroll
                     for (int r = 0; r < kRows; ++r) {
-                        const cplx<R> g = G[r][e];
+                        const cplx<R> g = gs.g[r];
                         const R p = g.re * X.re, q = g.im * X.im;
                         const R tr = p - q;            // Re(g X): node i
                         const R tl = p + q;            // Re(g conj X): node nx-1-i
@@ -158,8 +181,8 @@ tribo_status eval_impl(tribo_ctx* c, double t, void* dst) {
                      (const double*)c->d_damp, t, (cplx<R>*)c->d_mode_c);
     TRIBO_LAUNCHED(c);
     phase_begin(c, PH_FIELD);
-    (void)launch_pdl(k_mode_eval<R>, dim3((c->nz + kRows - 1) / kRows, rows), dim3(kEvalThreads), 0, c->stream, c->nx,
-                     rows, c->nz, nm, (const int2*)c->d_mode_a, (const double*)c->d_mode_f, (const cplx<R>*)c->d_mode_c,
+    (void)launch_pdl(k_mode_eval<R>, dim3((c->nz + kRows - 1) / kRows, rows), dim3(kEvalThreads), eval_smem<R>(c->nx),
+                     c->stream, c->nx, rows, c->nz, nm, (const int2*)c->d_mode_a, (const double*)c->d_mode_f, (const cplx<R>*)c->d_mode_c,
                      (const cplx<R>*)c->d_tabx, (const cplx<R>*)c->d_tabz, (const double*)c->d_ubar, (R*)dst);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
