@@ -17,7 +17,9 @@
 // sort's ping-pong between the particle sets ends where it started) and the
 // graph is replayed; remaining steps run as direct launches of the same work.
 // The step arguments live in device memory, so a captured graph stays valid
-// while the particle arrays stay the same (dt and parameters may change).
+// while the particle arrays (if it sorts them) and each channel's electrostatics
+// switch stay the same (dt and the other parameters may change); else it is
+// captured again.
 // The block size, tile size and grid of the particle kernel are picked by
 // timing candidates on scratch copies of the particles (tribo_batch_autotune).
 #include <algorithm>
@@ -400,10 +402,20 @@ tribo_status step_impl(tribo_batch* b, const std::vector<PView>& home, const dou
     }
     // while the particle kernel is timed every step is a direct launch
     if (left >= G && !b->timing) {
+        // what the graph holds by value: the sort kernels every array of a channel's particles (and by
+        // their alignment which gather; the particle kernel reads them from d_chans), the branches which
+        // channels solve
         std::vector<uintptr_t> key;
-        for (const PView& v : home) {
-            key.push_back((uintptr_t)v.x); key.push_back((uintptr_t)v.n); key.push_back((uintptr_t)v.id);
-            key.push_back((uintptr_t)v.site);
+        for (int i = 0; i < b->n; ++i) {
+            const PView& v = home[i];
+            if (b->sort_every > 0)
+                for (const void* a : {(const void*)v.x, (const void*)v.y, (const void*)v.z, (const void*)v.vx,
+                                      (const void*)v.vy, (const void*)v.vz, (const void*)v.d, (const void*)v.q,
+                                      (const void*)v.q_wall, (const void*)v.n_imp, (const void*)v.id,
+                                      (const void*)v.site})
+                    key.push_back((uintptr_t)a);
+            key.push_back((uintptr_t)v.n);
+            key.push_back((uintptr_t)(b->ch[i]->P.electrostatics != 0));
         }
         key.push_back((uintptr_t)G);
         key.push_back((uintptr_t)b->shape.nt * 1000003u + b->shape.tile * 31u + b->shape.bps);
