@@ -363,6 +363,10 @@ k_ysolve_twist(cplx<float>* __restrict__ S, cplx<float>* __restrict__ F, const f
                 const ds pt = h0 == 0 ? P[0][m] : po[m], pb = h0 == 0 ? po[m] : P[0][m];
                 xk[m] = ds_mul(ds_sub_mul(ds_sub_mul(m ? rk.y : rk.x, ek, pt), fk, pb), g);
             }
+        }
+        // both lanes of a pencil have read row k before one of them stores it
+        if constexpr (NH == 1) __syncwarp();
+        if (live) {
             if (h0 == 0) Sv[s0 + (uint32_t)k * rs] = make_float2(ds_f(xk[0]), ds_f(xk[1]));
 #pragma unroll
             for (int hh = 0; hh < NH; ++hh) {

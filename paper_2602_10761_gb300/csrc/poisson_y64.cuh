@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(128) k_ysolve64(cplx<R>* __restrict__ S, cplx<
         if (H > 0) xn = fma(-cpl[j0 + (H - 1) * dj], xk, P) * ip[(H - 1) * ts];
     }
     const double xo = __shfl_xor_sync(0xffffffffu, xn, 16);   // the other half's row next to k
+    __syncwarp();                            // both halves have read row k before one of them stores it
     if (!live) return;
     if (h == 0) srow[k * rs] = (R)xk;
     // substitution outwards; the E_y of a row one row behind it (the bottom half leaves row k to the top)
