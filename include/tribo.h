@@ -368,8 +368,10 @@ const char*  tribo_phase_name(int32_t phase);
  * and e.g. 256 x 64 x 64 in TRIBO_MIXED fits without phi (28.6 MiB) but not
  * with it (32.8 MiB).  A grid whose transforms need more shared memory per
  * block than the device offers is rejected with TRIBO_ERR_UNSUPPORTED.  The
- * first call on a device looks up that array's address (so make it before any
- * stream capture).  Calls share the array: calls whose GPU work overlaps race. */
+ * first call on a device looks up that array's address and loads the kernels of
+ * every grid and both precisions (so make it before any stream capture); later
+ * calls set nothing up, whatever their grid.  Calls share the array: calls whose
+ * GPU work overlaps race. */
 tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps, int32_t precision,
                                    const double* rho, double* phi, void* E, void* stream);
 

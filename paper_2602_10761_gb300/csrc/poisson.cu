@@ -22,7 +22,6 @@
 #include <cstring>
 #include <algorithm>
 #include <mutex>
-#include <set>
 
 #include "poisson_y64.cuh"
 #include "tribo_internal.cuh"
@@ -116,7 +115,7 @@ tribo_status poisson_free(tribo_ctx* c) {
 // device's memory, a real-time loop where an allocation's latency or failure
 // mid-run is not acceptable, or a plug-in that is only ever handed
 // pre-allocated buffers.  This variant keeps its scratch (coefficient tables,
-// twiddles, spectra, Thomas sweep storage) in one fixed file-scope device
+// twiddles, y factors, spectra) in one fixed file-scope device
 // array instead of a context's allocations.  It has no counterpart in the
 // paper.  Its tables are written into the array by its first kernel, from the
 // grid passed by value, so nothing is staged in or copied from host memory.
@@ -125,8 +124,11 @@ tribo_status poisson_free(tribo_ctx* c) {
 // the library holds it until the process exits.  Host code cannot use the
 // array's name as a device address, so the first call on each device (with
 // that device current) looks the address up once with cudaGetSymbolAddress
-// and keeps it; that first call should therefore come before any stream
-// capture.  All calls share the array and it keeps the last call's contents:
+// and keeps it; it also loads the kernels of every transform length and both
+// precisions (16 ms more than those of one grid), since code that CUDA loads at a
+// kernel's first launch takes device memory then.  That first call should
+// therefore come before any stream capture; later ones set nothing up, whatever
+// their grid.  All calls share the array and it keeps the last call's contents:
 // each call rewrites every byte it reads before reading it, and two calls
 // whose work overlaps on the GPU (different streams or devices sharing
 // nothing but this array on one device) race with each other.
@@ -141,10 +143,8 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratch
 
 struct NoallocDevice {
     unsigned char* base = nullptr;
-    int smem_max = 0;            // opt-in shared memory per block of the device
     int num_sms = 1;
     bool ready = false;
-    std::set<int> lengths;       // (precision, x or z, length) whose shared-memory limits are set
 };
 NoallocDevice g_noalloc_dev[kNoallocMaxDevices];
 std::mutex g_noalloc_mutex;
@@ -331,10 +331,26 @@ bool noalloc_2a3b(int n) {
     return n == 1;
 }
 
-// set-up of the current device: the array's device address, and the shared-memory limits of the
-// transforms of a grid when its lengths are first used
+// the kernels of one precision on the current device: the shared-memory limits of the transforms of
+// every length a grid may have (which loads their code: loaded when first launched, each would take
+// device memory then), and the code of the other two
 template <class R>
-tribo_status noalloc_device(int dev, int m, int nz, NoallocDevice* out) {
+tribo_status noalloc_load(int optin) {
+    tribo_status st;
+    for (int n = 4; n <= kNoallocMaxN; ++n) {
+        if (!noalloc_2a3b(n)) continue;
+        if (n % 2 == 0 && (st = xpass_attr<R>(n / 2, optin))) return st;
+        if ((st = zpass_attr<R>(n, optin))) return st;
+    }
+    cudaFuncAttributes at;
+    cudaError_t e = cudaFuncGetAttributes(&at, k_noalloc_tables<R>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, k_ysolve64<R>);
+    return e == cudaSuccess ? TRIBO_OK : cuda_fail(e, "tribo_poisson_noalloc: kernel attributes");
+}
+
+// set-up of the current device, by its first call: the array's device address and every kernel that a
+// later call of either precision may launch
+tribo_status noalloc_device(int dev, NoallocDevice* out) {
     std::lock_guard<std::mutex> lock(g_noalloc_mutex);
     NoallocDevice& d = g_noalloc_dev[dev];
     if (!d.ready) {
@@ -345,23 +361,13 @@ tribo_status noalloc_device(int dev, int m, int nz, NoallocDevice* out) {
         e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return cuda_fail(e, "tribo_poisson_noalloc: device attribute");
+        tribo_status st;
+        if ((st = noalloc_load<float>(optin)) || (st = noalloc_load<double>(optin))) return st;
         d.base = static_cast<unsigned char*>(p);
-        d.smem_max = optin;
         d.num_sms = std::max(1, sms);
         d.ready = true;
     }
-    const int kx = (int)sizeof(R) * 4096 + m, kz = (int)sizeof(R) * 4096 + 2048 + nz;
-    tribo_status st;
-    if (!d.lengths.count(kx)) {
-        if ((st = xpass_attr<R>(m, d.smem_max))) return st;
-        d.lengths.insert(kx);
-    }
-    if (!d.lengths.count(kz)) {
-        if ((st = zpass_attr<R>(nz, d.smem_max))) return st;
-        d.lengths.insert(kz);
-    }
-    out->base = d.base;
-    out->num_sms = d.num_sms;
+    *out = d;
     return TRIBO_OK;
 }
 
@@ -419,7 +425,7 @@ extern "C" tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps
     }
     NoallocDevice d;
     const bool f64 = precision == TRIBO_FP64;
-    tribo_status st = f64 ? noalloc_device<double>(dev, nx / 2, nz, &d) : noalloc_device<float>(dev, nx / 2, nz, &d);
+    tribo_status st = noalloc_device(dev, &d);
     if (st) return st;
     cudaStream_t s = (cudaStream_t)stream;
     if (f64) return noalloc_solve<double>(grid, eps, rho, phi, E, s, d.base, L, d.num_sms);

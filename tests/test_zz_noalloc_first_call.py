@@ -1,0 +1,71 @@
+"""The allocation-free solve's promise that only the first call on a device sets
+anything up, in a process of its own: after one mixed-precision call, calls with
+every other transform length and with the other precision leave the device's free
+memory as it was, and the first call of a new grid may come inside a stream capture.
+The captured solve's field is the one of the same call made directly."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SCRIPT = """
+import sys
+sys.path.insert(0, {root!r})
+import numpy as np
+import torch
+import paper_2602_10761_gb300 as T
+T.load()
+LENGTHS = sorted(2 ** a * 3 ** b for a in range(9) for b in range(6) if 4 <= 2 ** a * 3 ** b <= 256)
+assert len(LENGTHS) == 25
+
+def args(nx, ny, nz, prec):
+    real = torch.float64 if prec == T.TRIBO_FP64 else torch.float32
+    rho = torch.ones((nz, ny, nx), dtype=torch.float64, device="cuda")
+    E = torch.full((3, nz, ny + 2, nx), float("nan"), dtype=real, device="cuda")
+    return nx, ny, nz, 0.1, 0.05, np.linspace(0.0, 0.04, ny + 1), 8.854e-12, prec, rho, None, E
+
+calls = []
+for i, nz in enumerate(LENGTHS):
+    nx = next(n for n in LENGTHS[i:] if n % 2 == 0)
+    calls += [args(nx, 5, nz, prec) for prec in (T.TRIBO_FP64, T.TRIBO_MIXED)]
+side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+T.tribo_poisson_noalloc(*args(64, 8, 64, T.TRIBO_MIXED))
+torch.cuda.synchronize()
+free = torch.cuda.mem_get_info()[0]
+if {capture}:
+    a = args(48, 5, 36, T.TRIBO_FP64)
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        T.tribo_poisson_noalloc(*a, stream=torch.cuda.current_stream())
+    graph.replay()
+    torch.cuda.synchronize()
+    got = a[-1].clone()
+    a[-1].fill_(float("nan"))
+    T.tribo_poisson_noalloc(*a)
+    torch.cuda.synchronize()
+    assert torch.isfinite(got).all() and torch.equal(got, a[-1])
+else:
+    for a in calls:
+        T.tribo_poisson_noalloc(*a)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free, a[:3] + (a[7],)
+    assert all(torch.isfinite(a[-1]).all() for a in calls)      # (torch's own allocations come after the loop)
+print("done")
+"""
+
+
+@pytest.mark.parametrize("capture", [False, True])
+def test_only_the_first_call_sets_up(capture):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2602_10761_gb300 import build
+    build.build()
+    r = subprocess.run([sys.executable, "-c", SCRIPT.format(root=ROOT, capture=capture)], capture_output=True, text=True,
+                       timeout=300)
+    assert r.returncode == 0 and "done" in r.stdout, r.stderr[-2000:]
