@@ -118,19 +118,19 @@ __device__ __forceinline__ void collide_pair(const PView& p, uint32_t n, uint32_
 // 400 FP64 operations: run where it is found, each pair held a warp of its own and an SM's FP64
 // pipe, one lane in 32 in use (23.5 us a launch).  So the block lists the pairs of its particles
 // in shared memory and works through the list with all its lanes: 14.0 us.
-constexpr int kCollideThreads = 512;
-constexpr int kCollidePer = 4 * kCollideThreads;      // particles a block looks at per round
+constexpr int kCollideThreads = 512;                  // at most; a block looks at 4 particles a thread per round
 template <class R>
 __global__ void __launch_bounds__(kCollideThreads) k_pp_collide(PView p, const uint32_t* __restrict__ partner,
                                                                 double rho_p, double k_e, double el, double eps,
                                                                 double phi_p) {
     pdl_wait();
-    __shared__ uint32_t list[2 * kCollidePer];
+    __shared__ uint32_t list[2 * 4 * kCollideThreads];
     __shared__ unsigned int count;
     if (threadIdx.x == 0) count = 0;
     __syncthreads();
-    const int64_t stride = (int64_t)gridDim.x * kCollidePer;
-    for (int64_t n0 = (int64_t)blockIdx.x * kCollidePer; n0 < p.n; n0 += stride) {
+    const unsigned per = 4 * blockDim.x;              // particles of a round
+    const int64_t stride = (int64_t)gridDim.x * per;
+    for (int64_t n0 = (int64_t)blockIdx.x * per; n0 < p.n; n0 += stride) {
         const int64_t n = n0 + 4 * threadIdx.x;
         uint32_t j[4] = {kNone, kNone, kNone, kNone};
         if (n + 4 <= p.n) {                           // one 16-byte load (n is a multiple of 4)
@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(kCollideThreads) k_pp_collide(PView p, const u
         __syncthreads();
         const unsigned int m = count;
         __syncthreads();
-        // a round adds at most kCollidePer, so the list is emptied when it could not take another
-        if (m > (unsigned)kCollidePer || n0 + stride >= p.n) {
+        // a round adds at most `per`, so the list is emptied when it could not take another
+        if (m > per || n0 + stride >= p.n) {
             for (unsigned int i = threadIdx.x; i < m; i += blockDim.x)
                 collide_pair<R>(p, list[i], partner[list[i]], rho_p, k_e, el, eps, phi_p);
             if (threadIdx.x == 0) count = 0;
@@ -167,8 +167,15 @@ tribo_status collide_impl(tribo_ctx* c, const PView& p, const uint32_t* members,
     TRIBO_LAUNCHED(c);
     const tribo_params& P = c->P;
     phase_begin(c, PH_AUX);
-    const int64_t blocks = std::min<int64_t>((p.n + kCollidePer - 1) / kCollidePer, (int64_t)c->num_sms);
-    (void)launch_pdl(k_pp_collide<R>, dim3((unsigned)blocks), dim3(kCollideThreads), 0, c->stream, p, (const uint32_t*)partner,
+    // Few particles in small blocks, up to two per SM, so that their pairs spread over the SMs; past
+    // 2 x 1024 particles a SM blocks of 512, one a SM, whose lists fill the lanes.  A step of 2000
+    // particles that all collide: 122 us in blocks of 512, 76 so; of 40,000: 136, 89; from 311,296
+    // particles on the same launch as before.
+    int threads = 64;
+    while (threads < kCollideThreads && p.n > (int64_t)2 * c->num_sms * 4 * threads) threads *= 2;
+    const int64_t blocks = std::min<int64_t>((p.n + 4 * threads - 1) / (4 * threads),
+                                             (int64_t)c->num_sms * (threads == kCollideThreads ? 1 : 2));
+    (void)launch_pdl(k_pp_collide<R>, dim3((unsigned)blocks), dim3(threads), 0, c->stream, p, (const uint32_t*)partner,
                      P.rho_p, P.k_e, 2.0 * (1.0 - P.mu_p * P.mu_p) / P.E_p, P.eps, P.phi_p);
     TRIBO_LAUNCHED(c);
     return TRIBO_OK;
