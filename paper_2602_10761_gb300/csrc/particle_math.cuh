@@ -355,15 +355,21 @@ __device__ __forceinline__ void phi12(double s, double& phi1, double& phi2) {
     }
 }
 
-// x^(2/5), x > 0, in FP64: a particle that meets a wall holds its warp for the length of this chain,
-// so it is kept short.  y0 = x^(2/5) to FP32 accuracy; with e = x^2 / y0^5 - 1 (about 1e-6),
-// x^(2/5) = y0 (1 + e)^(1/5) = y0 (1 + e/5 - 2 e^2/25 + O(e^3)), the cube below 1e-17.
+// x^0.4, x > 0, in FP64: a particle that meets a wall holds its warp for the length of this chain,
+// so it is kept short.  y is x^(2/5) to FP32 accuracy; with e = x^2 / y^5 - 1 (up to 2e-5 at the ends of
+// the range), x^(2/5) = y (1 + e)^(1/5) = y (1 + e/5 - 2 e^2/25 + 6 e^3/125 - O(e^4)), the fourth power
+// below 1e-20.  The double 0.4, the exponent of the oracle, of the adjoint's pow and of the SSM's
+// reference area, is 2/5 + 2.22e-17, which makes x^0.4 a factor 1 + 1.54e-17 log2 x of it (1.5e-15 at
+// the ends).  Both corrections past e/5 are small enough for FP32.  Within 2.5e-16 of x^0.4.
 __device__ __forceinline__ double pow04(double x) {
     if (!(x > 1e-30 && x < 1e30)) return pow(x, 0.4);
-    const double y = (double)exp2f(0.4f * log2f((float)x));
+    const float l = log2f((float)x);
+    const double y = (double)exp2f(0.4f * l);
     const double y2 = y * y;
     const double e = x * x / (y2 * y2 * y) - 1.0;
-    return y + y * (e * (0.2 - 0.08 * e));
+    const float ef = (float)e;
+    const float t = ef * ef * (0.048f * ef - 0.08f) + 1.5391e-17f * l;
+    return y + y * (0.2 * e + (double)t);
 }
 // 1 - e^-x, x >= 0
 __device__ __forceinline__ double one_minus_exp(double x) {
@@ -376,7 +382,7 @@ __device__ __forceinline__ double one_minus_exp(double x) {
 }
 
 // the condenser-model charge of one wall impact (FP64) at the squared speed s2: with P = (alpha_coef
-// s2)^(2/5), alpha = r P and A = kappa_pi r alpha, so that A / (pi d^2) = kappa_pi P / (4 pi)
+// s2)^0.4, alpha = r P and A = kappa_pi r alpha, so that A / (pi d^2) = kappa_pi P / (4 pi)
 template <class R>
 __device__ __forceinline__ double impact_charge(const StepArgs<R>& a, double d, double s2, double q) {
     if (!(s2 > 0.0)) return 0.0;
