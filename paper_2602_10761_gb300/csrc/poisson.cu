@@ -189,7 +189,7 @@ NoallocLayout noalloc_layout(int nx, int ny, int nz, size_t rsz) {
 // reads host memory after it returns).
 struct NoallocGeom {
     int nx, ny, nz, n1;
-    double dx, dz, eps;
+    double dx, dz, scale;        // scale: -1 / (2 eps nx nz)
     double yf[kNoallocMaxN + 1];
 };
 
@@ -237,7 +237,8 @@ __global__ void __launch_bounds__(128) k_noalloc_tables(NoallocGeom g, double* _
     double* scale = ey + 3 * (ny + 2);
     for (int j = threadIdx.x; j < 3 * ny; j += blockDim.x) T[j] = sy[j];
     for (int j = threadIdx.x; j < ny; j += blockDim.x) {
-        scale[j] = -1.0 / g.eps / ((double)nx * (double)nz);
+        if constexpr (sizeof(R) == 8) scale[j] = g.scale;
+        else reinterpret_cast<float2*>(scale)[j] = make_float2((float)g.scale, (float)(g.scale - (double)(float)g.scale));
         // E_y at lattice node jn = j + 1: cm phi[j-1] + c0 phi[j] + cp phi[j+1]
         double cm = 0, c0 = 0, cp = 0;
         if (j >= 1) {
@@ -286,7 +287,8 @@ tribo_status noalloc_solve(const tribo_grid* g, double eps, const double* rho, d
     const int nx = g->nx, ny = g->ny, nz = g->nz, nxh = nx / 2 + 1;
     NoallocGeom geom{};
     geom.nx = nx; geom.ny = ny; geom.nz = nz;
-    geom.dx = g->lx / nx; geom.dz = g->lz / nz; geom.eps = eps;
+    geom.dx = g->lx / nx; geom.dz = g->lz / nz;
+    geom.scale = -0.5 / eps / ((double)nx * (double)nz);
     geom.n1 = 1;
     for (int d = 1; d * d <= nx / 2; ++d)
         if ((nx / 2) % d == 0) geom.n1 = d;

@@ -119,7 +119,14 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
     // fills its twiddle table, so that the table's round trip overlaps the loads
     cplx<R> y[N1];
     if (live && r < N2) {
-        const R s = (R)0.5 * from_f64<R>(scale_row[line % ny]);
+        R s, s_lo = 0;               // the row's factor
+        if constexpr (sizeof(R) == 4) {
+            const float2 v = reinterpret_cast<const float2*>(scale_row)[line % ny];
+            s = v.x;
+            s_lo = v.y;
+        } else {
+            s = scale_row[line % ny];
+        }
         using V2 = std::conditional_t<sizeof(QT) == 8, double2, float2>;   // (x_2n, x_2n+1)
         V2* row = reinterpret_cast<V2*>(src) + (size_t)line * M;
         unsigned nz_mask = 0;        // which element pairs hold a nonzero sum
@@ -127,7 +134,9 @@ __global__ void __launch_bounds__(kThreads, xfwd_min_blocks<R, M>()) k_xfwd4(QT*
         for (int n1 = 0; n1 < N1; ++n1) {
             const V2 v = row[N2 * n1 + r];
             nz_mask |= is_nonzero(v.x) | is_nonzero(v.y) ? 1u << n1 : 0u;
-            y[n1] = cplx<R>{from_f64<R>(v.x) * s, from_f64<R>(v.y) * s};
+            const R a = from_f64<R>(v.x), b = from_f64<R>(v.y);
+            if constexpr (sizeof(R) == 4) y[n1] = cplx<R>{fmaf(a, s, a * s_lo), fmaf(b, s, b * s_lo)};
+            else y[n1] = cplx<R>{a * s, b * s};
         }
         if (zero_src) {
             // most cells hold no particle: only pairs with a nonzero sum are rewritten, so the

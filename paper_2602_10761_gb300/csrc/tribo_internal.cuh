@@ -92,8 +92,8 @@ struct tribo_ctx {
     // device grid tables (FP64 and rounded-up FP32 copies for exact compares)
     double* d_yf = nullptr;      // ny+1
     double* d_Y = nullptr;       // ny+2 lattice nodes
-    double* d_scale_q = nullptr; // ny: -1 / (eps V_j nx nz) (charge sum -> RHS, normalised)
-    double* d_scale_rho = nullptr; // ny: -1 / (eps nx nz) (density -> RHS)
+    double* d_scale_q = nullptr; // ny: -1 / (2 eps V_j nx nz) (charge sum -> RHS, normalised; mixed: two floats)
+    double* d_scale_rho = nullptr; // ny: -1 / (2 eps nx nz) (density -> RHS)
     double* d_xf = nullptr;      // nx+1, nz+1 FP64 faces i dx, k dz (FP64 mode)
     double* d_zf = nullptr;
     float* d_yf_up = nullptr;    // ny+1: smallest float >= yf
@@ -241,7 +241,7 @@ tribo_status cuda_fail(cudaError_t e, const char* what);
 template <class R>
 struct FastTab {
     void* src;                  // FP64 cell charge sums (forward x source)
-    const double* scale;        // per-row RHS factor
+    const double* scale;        // per-row RHS factors (two floats each)
     cplx<R>* S;                 // spectrum
     cplx<R>* F;                 // field spectra (the E_y spectrum at F + fstride)
     R* E;                       // field lattice
@@ -282,7 +282,7 @@ tribo_status poisson_setup(tribo_ctx* c);
 tribo_status poisson_free(tribo_ctx* c);
 // src: device (nz, ny, nx) of doubles (src_f64: the FP64 cell charge sums or a
 // caller's FP64 density) or of the real type (the adjoint's charge adjoint);
-// scale: device ny per-row factor giving the RHS -rho/eps over nx nz; zero_src: write
+// scale: device ny per-row factors, the context's d_scale_q or d_scale_rho; zero_src: write
 // zeros back into src after reading.  phi may be NULL.  E: (3, nz, ny+2, nx)
 // real (E_x, E_y, E_z), or NULL for the potential alone (phi then non-NULL).
 tribo_status poisson_solve(tribo_ctx* c, void* src, bool src_f64, const double* scale, bool zero_src,
