@@ -361,17 +361,19 @@ const char*  tribo_phase_name(int32_t phase);
  * values passed by value, so the call copies nothing from host memory and
  * does not wait for earlier work on the stream.  All scratch lives in one
  * static device array of 32 MiB that the library reserves on every device it
- * is loaded on until the process exits.  Grids that need more, or more than
- * 256 cells in any direction, are rejected with TRIBO_ERR_CAPACITY
- * (tribo_last_error gives the sizes); the largest cubes that fit are 96^3 in
- * TRIBO_MIXED (27.9 MiB with phi) and 72^3 in TRIBO_FP64 (19.4 MiB with phi),
- * and e.g. 256 x 64 x 64 in TRIBO_MIXED fits without phi (28.6 MiB) but not
- * with it (32.8 MiB).  A grid whose transforms need more shared memory per
- * block than the device offers is rejected with TRIBO_ERR_UNSUPPORTED.  The
- * first call on a device looks up that array's address and loads the kernels of
- * every grid and both precisions (so make it before any stream capture); later
- * calls set nothing up, whatever their grid.  Calls share the array: calls whose
- * GPU work overlaps race. */
+ * is loaded on until the process exits.  A grid counts as its spectrum, three
+ * field spectra (four with phi), 24 bytes per row of every (m_x, m_z) pencil
+ * and its tables; grids that count as more than the array (the solve itself uses
+ * less), or with more than 256 cells in any direction, are rejected with
+ * TRIBO_ERR_CAPACITY (tribo_last_error gives the count); the largest cubes
+ * within it are 96^3 in TRIBO_MIXED (27.9 MiB with phi) and 72^3 in TRIBO_FP64
+ * (19.4 MiB with phi), and e.g. 256 x 64 x 64 in TRIBO_MIXED is accepted without
+ * phi (28.6 MiB) but not with it (32.8 MiB).  A grid whose transforms need more
+ * shared memory per block than the device offers is rejected with
+ * TRIBO_ERR_UNSUPPORTED.  The first call on a device looks up that array's
+ * address and loads the kernels of every grid and both precisions (so make it
+ * before any stream capture); later calls set nothing up, whatever their grid.
+ * Calls share the array: calls whose GPU work overlaps race. */
 tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps, int32_t precision,
                                    const double* rho, double* phi, void* E, void* stream);
 

@@ -151,8 +151,10 @@ std::mutex g_noalloc_mutex;
 
 size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 
-// The scratch that decides which grids the call takes: spectrum, nf field spectra and 24 bytes per
-// pencil and row of sweep storage beside the tables.
+// The rule by which the call takes a grid, part of its interface: the bytes that a spectrum, nf field
+// spectra and 24 bytes per pencil and row beside the tables come to may not exceed the array.  It is
+// an upper bound of the layout below (at most 26.7 MiB for every grid it lets through) and stays, so
+// that what the call refuses does not depend on how the solve uses the array.
 size_t noalloc_capacity(int nx, int ny, int nz, int nf, size_t rsz) {
     const size_t csz = 2 * rsz;
     const int nxh = nx / 2 + 1;
@@ -162,9 +164,8 @@ size_t noalloc_capacity(int nx, int ny, int nz, int nf, size_t rsz) {
            round256((size_t)ny * nz * nxh * (sizeof(double2) + sizeof(double)));
 }
 
-// What the passes use of it: the y tables (2 ny + 1 rows of (nz/2+1) nxh doubles) take the place of
-// the sweep storage and are smaller for every nz >= 4, the x twiddles carry their inner table, the
-// potential needs no field of its own.
+// What the solve uses of the array: tables, twiddles (x: with their inner table), y factors (2 ny + 1
+// rows of (nz/2+1) nxh doubles), the spectrum and three field spectra (the potential needs none).
 struct NoallocLayout {
     size_t tables, twx, twz, te, S, F, total;
 };
@@ -397,15 +398,15 @@ extern "C" tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps
         return TRIBO_ERR_UNSUPPORTED;
     }
     const size_t rsz = precision == TRIBO_FP64 ? sizeof(double) : sizeof(float);
-    const size_t need = noalloc_capacity(nx, ny, nz, phi ? 4 : 3, rsz);
+    const size_t counted = noalloc_capacity(nx, ny, nz, phi ? 4 : 3, rsz);
     const NoallocLayout L = noalloc_layout(nx, ny, nz, rsz);
-    if (nx > kNoallocMaxN || ny > kNoallocMaxN || nz > kNoallocMaxN || need > kNoallocScratchBytes ||
+    if (nx > kNoallocMaxN || ny > kNoallocMaxN || nz > kNoallocMaxN || counted > kNoallocScratchBytes ||
         L.total > kNoallocScratchBytes) {
         char buf[256];
         snprintf(buf, sizeof buf,
-                 "tribo_poisson_noalloc: a %dx%dx%d grid needs %.1f MiB of static scratch; the limit is "
+                 "tribo_poisson_noalloc: a %dx%dx%d grid counts as %.1f MiB of static scratch; the limit is "
                  "%d MiB and %d cells per direction",
-                 nx, ny, nz, need / 1048576.0, (int)(kNoallocScratchBytes >> 20), kNoallocMaxN);
+                 nx, ny, nz, counted / 1048576.0, (int)(kNoallocScratchBytes >> 20), kNoallocMaxN);
         set_last_error(buf);
         return TRIBO_ERR_CAPACITY;
     }
