@@ -64,8 +64,9 @@ size_t eval_smem(int nx) { return sizeof(cplx<R>) * (size_t)(2 * nx + (2 * nx) /
 // Read from global memory the x factors, nxi values apart, kept the L1 data pipe as busy as the
 // arithmetic by their bank conflicts; they come from a padded copy in shared memory, found by a
 // multiplication instead of a division by float, with the rows' values side by side and four modes in
-// flight: 123 -> 108 us, the same sums in the same order.  (128 or 256 modes staged: 110-112; two in
+// flight (FP32): 123 -> 108 us, the same sums in the same order.  (128 or 256 modes staged: 110-112; two in
 // flight: 115; the factors mode by mode in a table of their own: 111 alone, but 135 within a step.)
+// FP64, bound by its pipe: two in flight (four at 32 x 64 x 256: 2374 us, two 2159, elsewhere equal).
 template <class R>
 __global__ void __launch_bounds__(kEvalThreads)
 k_mode_eval(int nx, int ny2, int nz, int nm, const int2* __restrict__ ma, const double* __restrict__ mf,
@@ -112,7 +113,8 @@ k_mode_eval(int nx, int ny2, int nz, int nm, const int2* __restrict__ ma, const 
             }
             __syncthreads();
             if (i < npair) {
-#pragma unroll 4
+                constexpr int kInFlight = sizeof(R) == 4 ? 4 : 2;
+#pragma unroll kInFlight
                 for (int e = 0; e < cnt; ++e) {
                     const unsigned v = (unsigned)(AX[e] * ii);
                     const cplx<R> X = sx[xpad((int)(v - __umulhi(v, magic) * (unsigned)n2x))];
