@@ -380,16 +380,16 @@ tribo_status tribo_poisson_noalloc(const tribo_grid* grid, double eps, int32_t p
 /* Batched ensemble: many independent channels (each made by tribo_init with
  * its own grid, gas lattice, parameters and max_particles >= its particle
  * count) advanced together, as in the paper's sweeps over Re_tau and particle
- * size (Sec. 4).  Every step forks one branch per channel (cell sort when
+ * size (Sec. 4).  Every step forks one branch per channel (sort when
  * due, Poisson solve and field) and joins in ONE persistent particle kernel
  * over all channels' particles; steps are captured into a CUDA graph and
- * replayed.  Mixed-precision channels that share a grid whose transform
- * lengths are compiled in solve together: each pass of their Poisson solves
- * is one launch over all of them.  The channels must share precision and device and use frozen
+ * replayed.  Mixed-precision channels that share a grid solve together: each
+ * pass of their Poisson solves is one launch over all of them.  The channels must share precision and device and use frozen
  * gas lattices (no tribo_set_modes).  While a batch exists, its channels must
  * not be stepped or solved (tribo_step, tribo_poisson, tribo_adjoint) on their
  * own concurrently with it: they share the channel's work arrays.  sort_every: re-sort each
- * channel's particles by cell every this many batch steps (0 = never).
+ * channel's particles every this many batch steps (0 = never), in the order of
+ * tribo_params' sort_every.
  * stream: a cudaStream_t (NULL = legacy default) on which the batch joins. */
 typedef struct tribo_batch tribo_batch;
 tribo_status tribo_batch_create(tribo_batch** out, int32_t n_channels, tribo_ctx* const* channels,

@@ -231,8 +231,8 @@ def tribo_set_momentum_source(ctx: int, F_s=None) -> None:
 
 
 def tribo_set_adjoint_memory(ctx: int, max_bytes: int = -1) -> None:
-    """Budget of the adjoint's kept forward fields: < 0 half of the free device
-    memory (default), 0 never keep them, > 0 at most that many bytes."""
+    """Budget of the adjoint's kept forward fields and states: < 0 half of the free
+    device memory (default), 0 never keep them, > 0 at most that many bytes."""
     check(load().tribo_set_adjoint_memory(ctx, int(max_bytes)), "tribo_set_adjoint_memory")
 
 

@@ -4,7 +4,7 @@
 // together.
 //
 // Per step:
-//   fork   one branch per channel (its own stream): the cell sort when due,
+//   fork   one branch per channel (its own stream): the sort when due,
 //          then the channel's Poisson solve and field (Sec. 2.2);
 //   join   one persistent particle kernel for ALL channels' particles:
 //          a fixed grid walks a global tile space in order, block b taking
@@ -46,7 +46,7 @@ k_step_batch(const BatchChan<R>* __restrict__ chans, const int64_t* __restrict__
     BatchChan<R>& sc = *reinterpret_cast<BatchChan<R>*>(raw);
     extern __shared__ unsigned int sh_hist[];
     // the resident wave walks the tile space in order (block b takes tiles b, b + G, ...): the
-    // particles of a channel are cell-ordered, so the lattice the wave gathers from stays
+    // particles of a channel are ordered by node cell, so the lattice the wave gathers from stays
     // small in L2 (contiguous ranges per block spread the wave over every channel at once)
     (void)tiles_per_block;
     int cur = -1;
@@ -154,8 +154,8 @@ struct tribo_batch {
     int graph_steps = 0;
     int64_t graph_kernels = 0;
     int64_t launches = 0;
-    // channels solved together: groups of mixed-precision channels with one compiled-length
-    // grid (each split pass one launch over the group), and each channel's group (-1: alone)
+    // channels solved together: groups of mixed-precision channels with one grid (each split pass
+    // one launch over the group), and each channel's group (-1: alone)
     std::vector<void*> groups;
     std::vector<std::vector<int>> members;
     std::vector<int> group_of;
@@ -303,7 +303,7 @@ tribo_status issue_steps(tribo_batch* b, const std::vector<PView>& home, int cou
 template <class R>
 tribo_status autotune_impl(tribo_batch* b, const std::vector<PView>& home, const double* dt, int32_t* choice) {
     // scratch copies of the particles in the contexts' second sets; a channel that sorts is
-    // timed on a cell-sorted copy, the order it steps in (unsorted particles favour other shapes)
+    // timed on a sorted copy, the order it steps in (unsorted particles favour other shapes)
     std::vector<PView> scratch(b->n);
     for (int i = 0; i < b->n; ++i) {
         tribo_ctx* c = b->ch[i];
@@ -562,7 +562,7 @@ tribo_status tribo_batch_create(tribo_batch** out, int32_t n_channels, tribo_ctx
         destroy_batch(b);
         return st;
     }
-    // Poisson groups: two or more mixed-precision channels on one compiled-length grid
+    // Poisson groups: two or more mixed-precision channels on one grid
     b->group_of.assign(n_channels, -1);
     for (int i = 0; i < n_channels; ++i) {
         tribo_ctx* c = channels[i];

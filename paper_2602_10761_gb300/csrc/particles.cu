@@ -49,8 +49,8 @@ __global__ void __launch_bounds__(kStepThreads, step_min_blocks<R>()) k_step(Ste
     }
     unsigned int err = 0;
     // one resident wave of blocks walks the particles in windows of gridDim.x * blockDim.x: the
-    // particles are ordered by cell, so the lattice the wave gathers from stays small in L2.  The
-    // walk runs from the last cell plane down: the field pass wrote those planes last (they are
+    // particles are ordered by node cell, so the lattice the wave gathers from stays small in L2.  The
+    // walk runs from the last plane down: the field pass wrote those planes last (they are
     // still in L2), and the charge sums deposited last are the ones the next solve reads first
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t m = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; m < p.n; m += stride)
@@ -143,7 +143,7 @@ tribo_status deposit_impl(tribo_ctx* c, const PView& p) {
     return TRIBO_OK;
 }
 
-// ---------------------------------------------------------------- sort by cell
+// ---------------------------------------------------------------- sort and cell lists
 // Counting sort on a cell key: count (the atomic's return value is the
 // particle's rank inside its cell), exclusive scan of the counts over all
 // cells, the inverse permutation (slot offset[key] + rank takes the
@@ -157,7 +157,7 @@ __device__ __forceinline__ int node_below(R s, int n) {
     return i < 0 ? n - 1 : min(i, n - 1);
 }
 
-// kNode: the key is the node cell instead (the eight lattice nodes of the gather, cells shifted by
+// kNode (the re-sort): the key is the node cell instead (the eight lattice nodes of the gather, cells shifted by
 // half a spacing; the rows of the top cell's two halves share one key), the order the particle step
 // wants: it is bound by the sectors and cache lines its 48 gathers touch (ncu at 128^3, 1M particles:
 // L1 data pipe 84% busy, 15 sectors a load), and a warp of particles in node cell order reads one

@@ -3,7 +3,7 @@
 // Gauss-linear E_y and central E_x, E_z; the discretisation is described in
 // poisson.cu).  Every supported length 2^a 3^b has compiled transforms and
 // tabulated y factors (the field of a 288 x 145 x 162 grid in mixed precision:
-// 201 us; 1167 us with shared-memory Stockham passes and an FP64 Thomas sweep
+// 160 us; 1167 us with shared-memory Stockham passes and an FP64 Thomas sweep
 // with a division per row):
 //  * the x transforms are real: a length-nx/2 complex FFT of the packed line
 //    plus the split step (half the work and shared memory);

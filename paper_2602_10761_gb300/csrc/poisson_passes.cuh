@@ -52,7 +52,6 @@ __device__ __forceinline__ ds ds_mul(ds a, ds b) {
     e = fmaf(a.lo, b.hi, e);
     return fast_two_sum(p, e);
 }
-__device__ __forceinline__ ds ds_neg(ds a) { return {-a.hi, -a.lo}; }
 __device__ __forceinline__ float ds_f(ds a) { return a.hi + a.lo; }
 
 // ---------------------------------------------------------------- real transforms' split step
@@ -80,8 +79,10 @@ __device__ __forceinline__ cplx<R> split_inv_dx(cplx<R> xa, cplx<R> xb, cplx<R> 
 // transforms are in the scale), X_m and X_M-m from one sum and product.  Each thread zeroes the charge sums it has read.  The source has
 // type QT: the FP64 cell charge sums (or a caller's FP64 density), rounded to
 // R as they are read, or the adjoint's R-typed charge adjoint.
-// six resident blocks (40 registers) where the length fits them without spilling: FP32 factors up
-// to 16 (76 -> 75.8 us at 384x256x256); one otherwise
+// Bound by HBM.  Six resident blocks (40 registers) for FP32 factors up to 16 and M <= 192, one
+// otherwise: 85 us against 115 at 384x256x256, 37 against 44 at 288x145x162, 58 against 68 at 256^3,
+// although M = 192 and 144 spill 8 to 32 bytes so (the channel-table forms of 36 and 48 also 4 to 8).
+// M = 256, with the same factor, runs with one.
 template <class R, int M>
 constexpr int xfwd_min_blocks() { return sizeof(R) == 4 && M <= 192 && fft::FourStep<M, kThreads>::N2 <= 16 ? 6 : 1; }
 
@@ -236,7 +237,8 @@ __device__ __forceinline__ float ds_diff_f(ds a, ds b) { return (a.hi - b.hi) + 
 // bound by its instruction stream and its loads' latency together (51% issue,
 // 34% of stalls on loads before this form).  NH = 1: a pencil's halves run in two
 // lanes 16 apart and meet through shuffles; NH = 2: one thread runs both, two
-// interleaved chains.
+// interleaved chains, in 168 registers, six blocks a SM (with E_y it spills 60 bytes, the
+// channel-table form 72).
 // Which one: NH = 1 needs 128 registers for C = 6 rows ahead, four blocks of 64
 // pencils a SM; while the grid fits one such wave it is the faster (us, against
 // 64-pencil blocks of NH = 2, C = 5 at 168 registers): 128^3 24 / 32, 192x128x128

@@ -28,8 +28,8 @@ namespace {
 // value (E_y included), 21 us of the FP64 pipe at 128^3; the kernel it replaces
 // ran a |m_z| row's pencils in one thread (33 blocks at 128^3) with every row's
 // load exposed: 291 -> 40 us at 128^3, a 64^3 step 269 -> 146 us.  Its error
-// against an 80-bit solve is the one-sided sweep's (0.7 to 1.1 times it over
-// grids of 64 to 288 cells a side).
+// against an 80-bit solve is the one-sided sweep's but for scatter (phi 0.7 to
+// 1.3 times it, 1.0 in the mean over six grids and three seeds; E 1.0).
 // te: e_j (j <= k) and f_j (j > k), f_k at row ny; ti: i_j, g at row k.
 constexpr int kY64Rows = 8;                  // rows per chunk
 inline size_t ysolve64_smem(int ny) { return sizeof(double) * ((size_t)ny + 3 * (ny + 2)); }

@@ -119,8 +119,8 @@ struct tribo_ctx {
     void* S = nullptr;           // (nz, ny, nxh) cplx<real> spectrum
     void* F = nullptr;           // (4, nz, ny+2, nxh) cplx<real> field spectra
     // transform and y-solve tables (poisson_fast.cu)
-    void* d_ytab = nullptr;      // y-solve factors, rows of (nz/2+1)*nxh wavenumber pairs: FP64 ny+1 rows of
-                                 // couplings, ny of inverse pivots; mixed 2 x ny rows of float2
+    void* d_ytab = nullptr;      // y-solve factors, rows of (nz/2+1)*nxh wavenumber pairs: ny+1 rows of couplings,
+                                 // ny of inverse pivots, each a double or (mixed) a float2
     void* d_twx = nullptr;       // nx twiddles exp(-2 pi i e / nx), then the x transform's inner twiddles by thread
     void* d_twz = nullptr;       // nz twiddles
     void* d_ycpl = nullptr;      // ny float2: couplings of the y substitution in double-single (mixed mode)
@@ -325,7 +325,7 @@ struct StepIO {               // per-call overrides of the context's buffers
 tribo_status particles_step(tribo_ctx* c, const PView& p, double dt, bool deposit_next,
                             bool write_cell, const StepIO& io = StepIO());
 tribo_status particles_sum_q(tribo_ctx* c, const PView& p, double* d_out);
-// dst receives src sorted by cell key (all arrays; id if present)
+// dst receives src sorted by node cell (all arrays; id if present)
 tribo_status particles_sort(tribo_ctx* c, const PView& src, const PView& dst);
 tribo_status particles_setup(tribo_ctx* c);
 // per-cell lists of p (needs max_particles >= p.n): cell offsets in sort_counts,
